@@ -418,17 +418,18 @@ static int plan_grid(pq_ctx* ctx, int occ_index, int tiles_per_block = 8) {
 // stream is being captured: in a replayed graph the early blocks of the next
 // kernel were measured to slow the chain down.
 static thread_local bool t_chain = true;
+static thread_local size_t t_smem = 0;  // dynamic shared memory of the next launch
 template <typename... P, typename... A>
 static cudaError_t launch_chained(void (*k)(P...), int grid, int block, cudaStream_t s,
                                   A... args) {
   if (!t_chain) {
-    k<<<grid, block, 0, s>>>(args...);
+    k<<<grid, block, t_smem, s>>>(args...);
     return cudaGetLastError();
   }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(block);
-  cfg.dynamicSmemBytes = 0;
+  cfg.dynamicSmemBytes = t_smem;
   cfg.stream = s;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -492,7 +493,11 @@ pq_status launch_phase(pq_ctx* ctx, int phase, const Batch& b, bool vec, cudaStr
       e = launch_chained(k_plan_fscatter, plan_grid(ctx, 19, 1), 256, s, b);
       break;
     case kPhaseFagg: e = launch_chained(k_plan_fagg, plan_grid(ctx, 20, 1), 256, s, b); break;
-    case kPhaseF: e = launch_chained(k_plan_fprobe, plan_grid(ctx, 13), 256, s, b); break;
+    case kPhaseF:  // the direct pass's table of frequent groups, where it may run
+      t_smem = b.direct_ok ? sizeof(HotSums<kHotLog2>) : 0;
+      e = launch_chained(k_plan_fprobe, plan_grid(ctx, 13), 256, s, b);
+      t_smem = 0;
+      break;
     case kPhaseTopk: e = launch_chained(k_plan_topk, plan_grid(ctx, 7, 1), kTKW * 32, s, b); break;
   }
   prof_end(stop, s);
@@ -906,6 +911,10 @@ pq_status run_batch_internal(pq_ctx* ctx, const pq_plan* plans, int n, pq_result
     return cuda_fail(ctx, ue, "batch set-up");
   }
   Batch b = make_batch(ctx, ws, n, L);
+  // The direct F pass: one plan, resident columns, a static M bitmap whose
+  // rank records fit where the hit list would be.
+  b.direct_ok = n == 1 && !win && !any_part && descs[0].m_static && !descs[0].f_pair &&
+                direct_rec_bytes(descs[0].m_sb) <= (u64)al(descs[0].n_f * 4);
   b.clear_m = any_build ? 1 : 0;  // else no D scan runs: the memsets clear them
   if (!any_build) clears.insert(clears.end(), m_clears.begin(), m_clears.end());
 

@@ -350,6 +350,7 @@ struct Batch {
   PlanDev* q;
   int nq;
   int clear_m;    // the D scan clears the plans' static M bitmaps
+  int direct_ok;  // the batch's only plan may take the direct F pass
   const i64* tD;  // static tile prefixes [nq + 1]
   const i64* tM;
   const i64* tF;
@@ -369,6 +370,22 @@ enum { kPhDscan = 0, kPhDfill, kPhDbuild, kPhMscan, kPhMfill, kPhMbuild, kPhFpro
 constexpr int kMaxPartLog2 = 10;
 constexpr int kPT = 2048;
 constexpr int kAT = 1024;
+
+// The direct F pass (fdirect) takes a plan whose members are at least
+// one M row in kDirectShare: then enough F rows join that reading price and
+// discount with the key costs less than a hit list written, read back and
+// probed in a kernel of its own (10M clustered rows, all joining: the plan
+// 314 -> 173 us; the 60M-row plan of which 0.5 % join stays at 259 us).
+constexpr i64 kDirectShare = 8;
+// The M scan's verdict (Batch::direct_ok plans): a word of the work area, so
+// that the later kernels know it after a single load.
+constexpr int kDirectWord = 32;
+// Its rank records: per 32-bit word of the M bitmap the word and the number
+// of set bits before it, so that a rank is one 8-byte load.  They take the
+// place of the hit list.
+__host__ __device__ __forceinline__ u64 direct_rec_bytes(u64 bits) {
+  return (bits + 511) / 512 * 128;
+}
 
 // Bucket of a hit in a partitioned plan with 2^log2P buckets: the top bits
 // of its group slot among the plan's n slots, bucket = slot >> part_shift(n,
@@ -817,6 +834,7 @@ __device__ void mscan_finish(const Batch& b) {
   block_prefix(b.dyn + 2 * (b.nq + 1), b.nq, [&](int qi) -> i64 {
     const PlanDev& q = b.q[qi];
     if (q.m_static) {  // bitmap over the table's key range, set by this scan
+      if (b.direct_ok) b.work[kDirectWord] = ld_count(&q.ctr->mcount) >= q.n_m / kDirectShare;
       q.ctr->mlog2 = q.m_e;
       q.ctr->m_umin = q.m_su;
       q.ctr->m_bits = q.m_sb;
@@ -1385,6 +1403,25 @@ __global__ void __launch_bounds__(256) k_plan_mdup(Batch b) {
   const i64 total = pre[b.nq];
   const int lane = threadIdx.x & 31;
   const u64 keep = policy_keep();
+  if (b.direct_ok && b.work[kDirectWord]) {
+    // The direct pass's rank records, four words at a time (a tile's words
+    // are a multiple of 16).
+    const PlanDev& q = b.q[0];
+    const u64 bits = q.ctr->m_bits;
+    const DenseView dv = dense_view(q.ht_tag, (i64)q.ctr->mcount, bits);
+    const uint4* bm = reinterpret_cast<const uint4*>(dv.bm);
+    const uint2* wd = reinterpret_cast<const uint2*>(dv.wdir);
+    uint4* rec = reinterpret_cast<uint4*>(q.hlist);
+    const u64 quads = dv.blocks * 4;
+    for (u64 i = (u64)blockIdx.x * blockDim.x + threadIdx.x; i < quads;
+         i += (u64)gridDim.x * blockDim.x) {
+      const uint4 w = __ldcg(bm + i);
+      const uint2 p = __ldcg(wd + i);
+      const u32 t = __ldcg(dv.tdir + (i >> 8));  // 1024 words a tile
+      rec[2 * i] = make_uint4(w.x, t + (p.x & 0xFFFFu), w.y, t + (p.x >> 16));
+      rec[2 * i + 1] = make_uint4(w.z, t + (p.y & 0xFFFFu), w.w, t + (p.y >> 16));
+    }
+  }
   WarpClaim wc;
   while (true) {
     const i64 t = wc.next(b.work, kPhMdup);
@@ -1718,7 +1755,9 @@ __global__ void __launch_bounds__(256, 4) k_plan_fscan(Batch b) {
   u32* hr = s_hr[warp];
   const u64 keep = policy_keep(), strm = policy_stream();
   const bool ov = b.ov.table == 3;
-  const i64 total = ov ? b.ov.tiles : b.tF[b.nq];
+  // A plan that takes the direct pass leaves nothing to scan here.
+  const bool skip = !BUF && b.direct_ok && b.work[kDirectWord];
+  const i64 total = skip ? 0 : ov ? b.ov.tiles : b.tF[b.nq];
   int cq = -1;  // plan of the rows in the ring
   u32 hh = 0, ht = 0;
   auto flush = [&](u32 cnt) {  // cnt entries from hh to plan cq's hit list
@@ -1876,6 +1915,195 @@ __global__ void __launch_bounds__(256, 4) k_plan_fscan(Batch b) {
   }
 }
 
+// A block's table of the groups it meets often, direct-mapped.  A free entry
+// notes the last slot that came by and goes to the first that comes twice in
+// a row, which a frequent one does and a rare one hardly ever; from then on
+// its rows are added in shared memory.  A 64-bit sum is two 32-bit words whose
+// carries are passed on as they happen, so that the additions are native
+// shared-memory atomics; both words are exact modulo 2^64 whatever their
+// order.
+constexpr u32 kHotFree = 0xFFFFFFFFu;
+template <int LOG2>
+struct HotSums {
+  static constexpr int kN = 1 << LOG2;
+  u32 key[kN], lo[kN], hi[kN];
+  unsigned char last[kN];  // a few bits of the slot that came by last
+  __device__ void clear() {
+    for (int i = threadIdx.x; i < kN; i += blockDim.x)
+      key[i] = kHotFree, lo[i] = 0, hi[i] = 0, last[i] = 0;
+  }
+  __device__ __forceinline__ u32 owner(u32 slot) const {
+    return *(volatile const u32*)&key[(slot * 0x9E3779B1u) >> (32 - LOG2)];
+  }
+  // cur: owner(slot), read ahead.
+  __device__ __forceinline__ bool add(u32 slot, i64 v, u32 cur) {
+    const u32 p = slot * 0x9E3779B1u, h = p >> (32 - LOG2);
+    if (cur == kHotFree) {
+      // A race here loses or gains a candidate, never a row.
+      volatile unsigned char* const l = &last[h];
+      const unsigned char tag = (unsigned char)(p >> (24 - LOG2)) | 1;
+      if (*l != tag) {
+        *l = tag;
+        return false;
+      }
+      cur = atomicCAS(&key[h], kHotFree, slot);
+      if (cur == kHotFree) cur = slot;
+    }
+    if (cur != slot) return false;
+    const u32 a = (u32)(u64)v, old = atomicAdd(&lo[h], a);
+    const u32 up = (u32)((u64)v >> 32) + (old + a < old ? 1u : 0u);
+    if (up) atomicAdd(&hi[h], up);
+    return true;
+  }
+};
+
+// Direct F pass (run by the F probe kernel, so that other plans pay no launch
+// for it), for a plan whose rows mostly join (kDirectShare): one pass
+// over F tests the predicate, finds each row's group and adds its revenue.
+// No hit list.  A group is one 8-byte rank record (direct_rec_bytes); its sum
+// one reduction, or an addition in the block's table of frequent groups.  The
+// first-hit bit is set only by a row whose revenue is not positive: any other
+// group is known by its sum, which is then not zero (the top-k pass reads the
+// sums of all slots).  Where a sum might leave int64 (fast_commit does not
+// hold), each addition is checked and every row sets its bit.
+// A warp takes steps of 128 rows (lane l: rows 4l .. 4l+3), the grid's warps
+// consecutive ones; date is read two steps ahead, the other columns one.
+// What bounds it is random access: two per row (the record, the sum), where
+// the hit list, the two directories, the sum and the hit bit were six.  200M
+// rows over 40M groups (Zipf keys, 320 MB of sums, beyond L2: 12.9 GB of DRAM
+// traffic for 4.2 GB of columns): scan and probe 7.27 -> 3.23 ms; 50M rows
+// over 10M groups 1.2 -> 0.38 ms.  The table of frequent groups without its
+// second-visit rule: 4.7 ms; of 512 entries 5.5 ms; without it (one address
+// takes a reduction per 1.8 ns) 26 ms; of 4096 entries, which leave the L1
+// less room for the records, 4.4 ms.
+constexpr int kHotLog2 = 10;
+template <bool VEC>
+__device__ __forceinline__ void fdirect(const Batch& b, HotSums<kHotLog2>& hot) {
+  const PlanDev& q = b.q[0];
+  QCtr* const c = q.ctr;
+  hot.clear();
+  __syncthreads();
+  const int lane = threadIdx.x & 31;
+  const u64 keep = policy_keep(), strm = policy_stream();
+  const i64 n = q.n_f;
+  const i64* const mkey = q.f_mkey;
+  const i64* const price = q.f_price;
+  const signed char* const disc = q.f_disc;
+  const int* const date = q.f_date;
+  const Pred32 pf = to32(q.pf);
+  const u64 ubase = c->m_umin ^ 0x8000000000000000ULL, bits = c->m_bits;
+  const uint2* const rec = reinterpret_cast<const uint2*>(q.hlist);
+  const DenseLayout L = dense_layout((i64)c->mcount, bits);
+  char* const gb = reinterpret_cast<char*>(q.ht_tag);
+  u32* const hit = reinterpret_cast<u32*>(gb + L.hit);
+  i64* const sums = reinterpret_cast<i64*>(gb + L.sums);
+  const u32* const cnt = c->dup ? reinterpret_cast<const u32*>(gb + L.cnt) : nullptr;
+  const bool exact = !fast_commit(q, (u64)n);
+  const i64 steps = (n + 127) / 128, stride = (i64)gridDim.x * (blockDim.x >> 5);
+  const i64 s0 = (i64)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  auto ld_d = [&](i64 s) -> int4 {
+    const i64 r = s * 128 + 4 * lane;
+    return s < steps ? load_i32x4<VEC>(date, r, n - r, strm) : make_int4(0, 0, 0, 0);
+  };
+  auto p4 = [&](int4 d, i64 s) -> u32 {
+    return s < steps ? pass4(pf, d, n - (s * 128 + 4 * lane)) : 0u;
+  };
+  // Key, price and discount of a lane's 4 rows, when one of them passes.
+  auto ld_row = [&](i64 s, u32 m, i64 (&k)[4], i64 (&pr)[4], u32& ds) {
+    if (!m) return;
+    const i64 r = s * 128 + 4 * lane;
+    load_i64x4<VEC>(mkey, r, n - r, m, strm, k);
+    load_i64x4<VEC>(price, r, n - r, m, strm, pr);
+    if (VEC && n - r >= 4) {
+      ds = ld_stream(reinterpret_cast<const u32*>(disc + r));
+    } else {
+      ds = 0;
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        if ((m >> j) & 1u) ds |= (u32)(unsigned char)ld_stream(disc + r + j) << (8 * j);
+    }
+  };
+  i64 kA[4], pA[4];
+  u32 dA = 0;
+  int4 dB = ld_d(s0);
+  u32 mA = p4(dB, s0);
+  ld_row(s0, mA, kA, pA, dA);
+  dB = ld_d(s0 + stride);
+  u64 hits = 0;
+  for (i64 s = s0; s < steps; s += stride) {
+    // The rank records of this step's keys, then the next step's columns.
+    uint2 w[4];
+    u32 sh = 0, ok = 0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const u64 idx = (u64)kA[j] - ubase;
+      const bool in = ((mA >> j) & 1u) && idx < bits;
+      // Unconditional (the first record for rows that do not count), so that
+      // the four loads are in flight together.
+      asm("ld.global.nc.L2::cache_hint.v2.u32 {%0, %1}, [%2], %3;"
+          : "=r"(w[j].x), "=r"(w[j].y)
+          : "l"(rec + (in ? (u32)(idx >> 5) : 0u)), "l"(keep));
+      sh |= ((u32)idx & 31u) << (5 * j);
+      ok |= (u32)in << j;
+    }
+    const u32 mB = p4(dB, s + stride);
+    i64 kB[4], pB[4];
+    u32 ds = 0;
+    ld_row(s + stride, mB, kB, pB, ds);
+    dB = ld_d(s + 2 * stride);
+    u32 slot[4], live = 0;
+    i64 v[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const u32 bit = (sh >> (5 * j)) & 31u;
+      live |= ((w[j].x >> bit) & (ok >> j) & 1u) << j;
+      slot[j] = w[j].y + __popc(w[j].x & ((1u << bit) - 1u));
+      v[j] = pA[j] * (100 - (i64)(signed char)(dA >> (8 * j)));
+    }
+    hits += __popc(live);
+    if (exact) {
+#pragma unroll 1
+      for (int j = 0; j < 4; ++j) {
+        if (!((live >> j) & 1u)) continue;
+        const i64 pj = j == 0 ? pA[0] : j == 1 ? pA[1] : j == 2 ? pA[2] : pA[3];
+        const u32 sj = j == 0 ? slot[0] : j == 1 ? slot[1] : j == 2 ? slot[2] : slot[3];
+        const __int128 v128 = (__int128)(cnt ? (i64)__ldg(cnt + sj) : 1) *
+                              ((__int128)pj * (100 - (i64)(signed char)(dA >> (8 * j))));
+        const i64 vj = (i64)v128;
+        red_or(hit + (sj >> 5), 1u << (sj & 31));
+        const i64 old = (i64)atomicAdd((u64*)(sums + sj), (u64)vj);
+        if (v128 != (__int128)vj || add_overflows(old, vj))
+          q_latch(c, b.st, PQ_ERR_OVERFLOW, (i64)sj);
+      }
+    } else {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        if (!((live >> j) & 1u)) continue;
+        if (cnt) v[j] *= (i64)__ldg(cnt + slot[j]);
+        if (v[j] <= 0) red_or(hit + (slot[j] >> 5), 1u << (slot[j] & 31));
+      }
+      // Neighbouring rows of one group (clustered keys) are added once.
+#pragma unroll
+      for (int j = 0; j < 3; ++j)
+        if (((live >> j) & 3u) == 3u && slot[j] == slot[j + 1]) v[j + 1] += v[j], live &= ~(1u << j);
+      u32 own[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) own[j] = hot.owner(slot[j]);
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        if (((live >> j) & 1u) && !hot.add(slot[j], v[j], own[j])) red_add(sums + slot[j], v[j]);
+    }
+    mA = mB, dA = ds;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) kA[j] = kB[j], pA[j] = pB[j];
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < hot.kN; i += blockDim.x)
+    if (hot.key[i] != kHotFree) red_add(sums + hot.key[i], (i64)((u64)hot.hi[i] << 32 | hot.lo[i]));
+  const u32 h = __reduce_add_sync(kFull, (u32)hits);  // a warp's rows: below 2^32
+  if (lane == 0 && h) atomicAdd(&c->hits_total, (u64)h);
+}
+
 // F probe: warp tiles of the hit list (hp_tile rows), 32 per batch: each
 // lane re-reads its row's key, price and discount, finds the group (dense:
 // rank of the key's bit; hash: probe), and the batch commits (lanes of the
@@ -1883,11 +2111,17 @@ __global__ void __launch_bounds__(256, 4) k_plan_fscan(Batch b) {
 // memory).  A plan with at least 2048 hits per block of the grid (skewed or
 // pass-all data, where groups repeat within a block) first tries the
 // block's shared aggregation table.
-__global__ void __launch_bounds__(256) k_plan_fprobe(Batch b) {
+__global__ void __launch_bounds__(256, 4) k_plan_fprobe(Batch b) {
   chain_begin();
   __shared__ u64 s_akey[kAgg];
   __shared__ i64 s_asum[kAgg];
   __shared__ i64 s_sc[8][32];
+  extern __shared__ __align__(16) unsigned char s_dyn[];  // only when direct_ok
+  if (b.direct_ok && b.work[kDirectWord]) {
+    auto& hot = *reinterpret_cast<HotSums<kHotLog2>*>(s_dyn);
+    if (b.q[0].vec) fdirect<true>(b, hot);
+    else fdirect<false>(b, hot);
+  }
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   i64* sc = s_sc[warp];
   for (int i = threadIdx.x; i < kAgg; i += blockDim.x) s_akey[i] = 0, s_asum[i] = 0;
@@ -2257,11 +2491,13 @@ struct TopkSrc {
   const longlong2* rec;
   const i64* sums;
   i64 words;
+  i64 slots;  // dense slots
   bool dense;
 };
 __device__ __forceinline__ TopkSrc topk_src(const PlanDev& q) {
   TopkSrc t;
   t.dense = q.ctr->m_bits != 0;
+  t.slots = (i64)q.ctr->mcount;
   if (t.dense) {
     const DenseLayout L = dense_layout((i64)q.ctr->mcount, q.ctr->m_bits);
     const char* base = reinterpret_cast<const char*>(q.ht_tag);
@@ -2343,6 +2579,125 @@ __device__ __forceinline__ u64 tk_scan(const TopkSrc& src, i64 tw, i64 lt, u32* 
   return groups;
 }
 
+// tk_scan for the groups of the direct pass: every slot of the tile is read,
+// 512 at a time, the next 512 while these are looked at.  Slots whose sum is
+// below `least` are only counted; the others go through the ring to on(KS),
+// 256 at a time.
+template <typename On>
+__device__ __forceinline__ u64 tk_scan_sums(const TopkSrc& src, i64 tw, i64 lt, i64 least,
+                                            u32* ring, On on) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const i64 ww = tw / kTKW;
+  const i64 w0 = lt * tw + warp * ww, w1 = min(src.words, w0 + ww);
+  longlong2 x[8];
+  u32 hw = 0;
+  auto load = [&](i64 w) {
+    const i64 s0 = w * 32 + 2 * lane;
+    // Whole steps load without conditions: with them each load was waited
+    // for before the next was issued (8800 cycles a step instead of 2450).
+    if (w + 16 <= w1 && (w + 16) * 32 <= src.slots) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+        x[i] = __ldcg(reinterpret_cast<const longlong2*>(src.sums + s0 + i * 64));
+    } else {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const i64 s = s0 + i * 64;
+        const bool in = w + 2 * i + (lane >> 4) < w1;
+        x[i].x = in && s < src.slots ? __ldcg(src.sums + s) : 0;
+        x[i].y = in && s + 1 < src.slots ? __ldcg(src.sums + s + 1) : 0;
+      }
+    }
+    hw = lane < 16 && w + lane < w1 ? __ldcg(src.hit + w + lane) : 0u;
+  };
+  u32 head = 0, tail = 0;
+  auto drain = [&](u32 cnt) {  // cnt <= 256 entries from head
+    KS r[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const u32 j = u * 32 + lane;
+      const u32 slot = j < cnt ? ring[(head + j) & (kTKR - 1)] : 0u;
+      r[u].k = slot, r[u].s = j < cnt ? __ldcg(src.sums + slot) : 0, r[u].v = j < cnt;
+    }
+    on(r);
+    head += cnt;
+    __syncwarp();
+  };
+  u64 groups = 0;
+  if (w0 < w1) load(w0);
+  for (i64 w = w0; w < w1; w += 16) {
+    u32 live = 0, top = 0;  // bit 2i, 2i + 1: the lane's slots of group i
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      live |= ((__shfl_sync(kFull, hw, 2 * i + (lane >> 4)) >> (2 * (lane & 15))) & 3u) << (2 * i);
+      live |= (u32)(x[i].x != 0) << (2 * i) | (u32)(x[i].y != 0) << (2 * i + 1);
+      top |= (u32)(x[i].x >= least) << (2 * i) | (u32)(x[i].y >= least) << (2 * i + 1);
+    }
+    if (w + 16 < w1) load(w + 16);
+    groups += __popc(live);
+    top &= live;
+    if (!__any_sync(kFull, top)) continue;
+    const u32 c = __popc(top);
+    u32 incl = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const u32 y = __shfl_up_sync(kFull, incl, o);
+      if (lane >= o) incl += y;
+    }
+    u32 pos = tail + incl - c;
+    for (; top; top &= top - 1) {
+      const int j = __ffs(top) - 1;
+      ring[pos++ & (kTKR - 1)] = (u32)(w * 32) + (j >> 1) * 64 + 2 * lane + (j & 1);
+    }
+    tail += __shfl_sync(kFull, incl, 31);
+    __syncwarp();
+    while (tail - head >= 256) drain(256);
+  }
+  if (tail != head) drain(tail - head);
+  return groups;
+}
+
+// A tile's top K over the groups of the direct pass.  With at least 32 slots
+// per thread a first threshold (the K-th best of the threads' best of 16
+// sampled slots) keeps all but a few records out of the lists: at least K
+// records are not below it.  Returns as tk_lane_rank (K <= 32).
+__device__ __forceinline__ int topk_tile_sums(const TopkSrc& src, i64 tw, i64 lt, int K, u32* ring,
+                                              LaneRankSmem<kTKW * 32>* lr, i64* tk, i64* ts,
+                                              u64* groups) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  i64 least = INT64_MIN;
+  if (tw >= 32 * kTKW) {  // block-uniform
+    const i64 b0 = (lt * tw + warp * (tw / kTKW)) * 32, nb = tw / kTKW * 32;
+    i64 hk = 0, hs = 0;
+#pragma unroll
+    for (int j = 0; j < 16; ++j) {
+      const i64 sl = b0 + nb / 16 * j + lane;
+      const i64 x = sl < src.slots ? __ldcg(src.sums + sl) : 0;
+      if (x != 0 && (hs == 0 || x > hs)) hk = sl, hs = x;
+    }
+    if (threadIdx.x == 0) lr->nh = 0, lr->found = 0;
+    __syncthreads();
+    int h = -1;
+    if (hs != 0) {
+      h = atomicAdd(&lr->nh, 1);
+      lr->hk[h] = hk, lr->hs[h] = hs;
+    }
+    __syncthreads();
+    if (hs != 0 && rank_among(lr->hk, lr->hs, lr->nh, hk, hs, h) == K - 1)
+      lr->ths = hs, lr->found = 1;
+    __syncthreads();
+    if (lr->found) least = lr->ths;
+    __syncthreads();  // tk_lane_rank reuses lr
+  }
+  LaneTop T;
+  T.clear();
+  *groups = tk_scan_sums(src, tw, lt, least, ring, [&](const KS* r) {
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (r[u].v) T.insert(r[u].k, r[u].s);
+  });
+  return tk_lane_rank(T, K, *lr, tk, ts);
+}
 // K rounds of the last tile's merge (one warp): lane l owns tiles l + 32 j
 // (j < kTKP / 32) and keeps their heads in registers; a round takes the best
 // head of the warp (warp max reductions over the record's order value, 32
@@ -2500,24 +2855,87 @@ __device__ __forceinline__ void topk_final(const PlanDev& q, int K, int parts, b
   }
 }
 
-__global__ void __launch_bounds__(kTKW * 32) k_plan_topk(Batch b) {
+// Shared memory of the top-k kernel.
+struct TopkSmem {
+  __align__(16) u32 ring[kTKW][kTKR];
+  i64 scr[kTKW][kTopScr];
+  i64 mk[kTKW * kMaxK], ms[kTKW * kMaxK];
+  int mc[kTKW];
+  LaneRankSmem<kTKW * 32> lr;
+  i64 t;
+  int cnt;
+  bool last;
+};
+
+// A tile's list is out: the block that finds itself last among the plan's
+// tiles merges them all (called by every thread of the block).
+__device__ __forceinline__ void topk_tile_done(const Batch& b, const PlanDev& q, i64 lt, int parts,
+                                               bool dense, u64 groups, TopkSmem& sm) {
+#pragma unroll
+  for (int o = 16; o; o >>= 1) groups += __shfl_xor_sync(kFull, groups, o);
+  if ((threadIdx.x & 31) == 0 && groups) atomicAdd(&q.ctr->gcount, groups);
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    q.tk_c[lt] = sm.cnt;
+    __threadfence();
+    sm.last = (int)atomicAdd(&q.ctr->tk_ticket, 1u) == parts - 1;
+    if (sm.last) fence_acq_rel_gpu();
+  }
+  __syncthreads();
+  if (!sm.last) return;
+  fence_acq_rel_gpu();  // the other tiles' lists, published before their tickets
+  topk_final(q, q.k, parts, dense, &sm.ring[0][0], b.st);
+}
+
+// The top-k of a plan that took the direct pass, in a function of its own so
+// that the other plans' top-k keeps its registers and fetches none of it.
+__device__ __noinline__ void topk_direct(const Batch& b, TopkSmem& sm) {
+  const PlanDev& q = b.q[0];
+  const int warp = threadIdx.x >> 5, K = q.k;
+  const TopkSrc src = topk_src(q);
+  const i64 tw = topk_tile_words_w(src.words);
+  const i64 parts = b.dyn[4 * (b.nq + 1) + b.nq];
+  for (i64 lt = blockIdx.x; lt < parts; lt += gridDim.x) {
+    i64* tk = q.cand_k + lt * K;
+    i64* ts = q.cand_s + lt * K;
+    u64 groups = 0;
+    int nres = -1;
+    if (K <= 32) nres = topk_tile_sums(src, tw, lt, K, sm.ring[warp], &sm.lr, tk, ts, &groups);
+    if (nres < 0) {  // K > 32, or the lanes' lists cannot vouch for it: per-warp lists
+      TopList L;
+      L.bind(sm.scr[warp]);
+      L.clear();
+      groups = tk_scan_sums(src, tw, lt, INT64_MIN, sm.ring[warp], [&](const KS* r) {
+#pragma unroll
+        for (int u = 0; u < 8; ++u) L.offer(K, r[u].v, r[u].k, r[u].s);
+      });
+      tk_block_merge_all(L, K, sm.mk, sm.ms, sm.mc);
+      if (warp == 0) L.store(tk, ts);
+      nres = L.cnt;
+    }
+    if (threadIdx.x == 0) sm.cnt = nres;
+    topk_tile_done(b, q, lt, (int)parts, true, groups, sm);
+    __syncthreads();  // sm is used again by the next tile
+  }
+}
+
+__global__ void __launch_bounds__(kTKW * 32, 4) k_plan_topk(Batch b) {
   chain_begin();
-  __shared__ __align__(16) u32 s_ring[kTKW][kTKR];
-  __shared__ i64 s_scr[kTKW][kTopScr];
-  __shared__ i64 s_mk[kTKW * kMaxK], s_ms[kTKW * kMaxK];
-  __shared__ int s_mc[kTKW];
-  __shared__ LaneRankSmem<kTKW * 32> s_lr;
-  __shared__ i64 s_t;
-  __shared__ int s_cnt;
-  __shared__ bool s_last;
+  __shared__ TopkSmem sm;
+  if (b.direct_ok && b.work[kDirectWord]) {
+    topk_direct(b, sm);
+    finish(b.work, kPhTopk);
+    return;
+  }
   const i64* pre = b.dyn + 4 * (b.nq + 1);
   const i64 total = pre[b.nq];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   TopList L;
-  L.bind(s_scr[warp]);
+  L.bind(sm.scr[warp]);
   BlockClaim bc;
   while (true) {
-    const i64 t = bc.next(b.work, kPhTopk, &s_t);
+    const i64 t = bc.next(b.work, kPhTopk, &sm.t);
     if (t >= total) break;
     const int qi = find_q(pre, b.nq, t);
     const PlanDev& q = b.q[qi];
@@ -2538,46 +2956,29 @@ __global__ void __launch_bounds__(kTKW * 32) k_plan_topk(Batch b) {
     if (K <= 32) {
       LaneTop T;
       T.clear();
-      groups = tk_scan(src, tw, lt, s_ring[warp], [&](const KS* r) {
+      groups = tk_scan(src, tw, lt, sm.ring[warp], [&](const KS* r) {
 #pragma unroll
         for (int u = 0; u < 8; ++u)
           if (r[u].v) T.insert(r[u].k, r[u].s);
       });
-      const int nres = tk_lane_rank(T, K, s_lr, tk, ts);
+      const int nres = tk_lane_rank(T, K, sm.lr, tk, ts);
       done = nres >= 0;
-      if (done && threadIdx.x == 0) s_cnt = nres;
+      if (done && threadIdx.x == 0) sm.cnt = nres;
     }
     if (!done) {
       L.clear();
-      const u64 g = tk_scan(src, tw, lt, s_ring[warp], [&](const KS* r) {
+      const u64 g = tk_scan(src, tw, lt, sm.ring[warp], [&](const KS* r) {
 #pragma unroll
         for (int u = 0; u < 8; ++u) L.offer(K, r[u].v, r[u].k, r[u].s);
       });
       if (K > 32) groups = g;
-      tk_block_merge_all(L, K, s_mk, s_ms, s_mc);
+      tk_block_merge_all(L, K, sm.mk, sm.ms, sm.mc);
       if (warp == 0) {
         L.store(tk, ts);
-        if (lane == 0) s_cnt = L.cnt;
+        if (lane == 0) sm.cnt = L.cnt;
       }
     }
-#pragma unroll
-    for (int o = 16; o; o >>= 1) groups += __shfl_xor_sync(kFull, groups, o);
-    if (lane == 0 && groups) atomicAdd(&q.ctr->gcount, groups);
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      q.tk_c[lt] = s_cnt;
-      __threadfence();
-      s_last = (int)atomicAdd(&q.ctr->tk_ticket, 1u) == parts - 1;
-      if (s_last) fence_acq_rel_gpu();
-    }
-    __syncthreads();
-    if (!s_last) {
-      if (gridDim.x >= total) break;
-      continue;
-    }
-    fence_acq_rel_gpu();  // the other tiles' lists, published before their tickets
-    topk_final(q, K, parts, src.dense, &s_ring[0][0], b.st);
+    topk_tile_done(b, q, lt, parts, src.dense, groups, sm);
     if (gridDim.x >= total) break;  // one tile per block: no ticket needed to stop
   }
   finish(b.work, kPhTopk);
