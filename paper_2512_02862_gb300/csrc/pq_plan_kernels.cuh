@@ -1915,48 +1915,6 @@ __global__ void __launch_bounds__(256, 4) k_plan_fscan(Batch b) {
   }
 }
 
-// A block's table of the groups it meets often, direct-mapped.  A free entry
-// notes the last slot that came by and goes to the first that comes twice in
-// a row, which a frequent one does and a rare one hardly ever; from then on
-// its rows are added in shared memory.  A 64-bit sum is two 32-bit words whose
-// carries are passed on as they happen, so that the additions are native
-// shared-memory atomics; both words are exact modulo 2^64 whatever their
-// order.
-constexpr u32 kHotFree = 0xFFFFFFFFu;
-template <int LOG2>
-struct HotSums {
-  static constexpr int kN = 1 << LOG2;
-  u32 key[kN], lo[kN], hi[kN];
-  unsigned char last[kN];  // a few bits of the slot that came by last
-  __device__ void clear() {
-    for (int i = threadIdx.x; i < kN; i += blockDim.x)
-      key[i] = kHotFree, lo[i] = 0, hi[i] = 0, last[i] = 0;
-  }
-  __device__ __forceinline__ u32 owner(u32 slot) const {
-    return *(volatile const u32*)&key[(slot * 0x9E3779B1u) >> (32 - LOG2)];
-  }
-  // cur: owner(slot), read ahead.
-  __device__ __forceinline__ bool add(u32 slot, i64 v, u32 cur) {
-    const u32 p = slot * 0x9E3779B1u, h = p >> (32 - LOG2);
-    if (cur == kHotFree) {
-      // A race here loses or gains a candidate, never a row.
-      volatile unsigned char* const l = &last[h];
-      const unsigned char tag = (unsigned char)(p >> (24 - LOG2)) | 1;
-      if (*l != tag) {
-        *l = tag;
-        return false;
-      }
-      cur = atomicCAS(&key[h], kHotFree, slot);
-      if (cur == kHotFree) cur = slot;
-    }
-    if (cur != slot) return false;
-    const u32 a = (u32)(u64)v, old = atomicAdd(&lo[h], a);
-    const u32 up = (u32)((u64)v >> 32) + (old + a < old ? 1u : 0u);
-    if (up) atomicAdd(&hi[h], up);
-    return true;
-  }
-};
-
 // Direct F pass (run by the F probe kernel, so that other plans pay no launch
 // for it), for a plan whose rows mostly join (kDirectShare): one pass
 // over F tests the predicate, finds each row's group and adds its revenue.

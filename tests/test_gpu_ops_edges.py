@@ -78,3 +78,136 @@ def test_filter_without_room_for_its_bits(stream):
     a = np.random.default_rng(5).integers(0, 100, size=9_000_001).astype(np.int32)
     check_filter(small, stream, a, "<", 37)
     small.close()
+
+
+def check_groupby(ctx, stream, k, v, cap=None, off=0):
+    want = oracle.groupby_sum(k[off:], v[off:])
+    cap = len(want[0]) if cap is None else cap
+    x, y = dev(k)[off:], dev(v)[off:]
+    torch.cuda.synchronize()
+    with torch.cuda.stream(stream):
+        ok, os_, ng = pq.pq_groupby_sum(ctx, x, y, cap=cap, stream=stream)
+        ctx.sync(stream)
+    g = int(ng.item())
+    assert g == len(want[0])
+    gk, gs = ok[:g].cpu().numpy(), os_[:g].cpu().numpy()
+    order, worder = np.argsort(gk), np.argsort(want[0])
+    assert np.array_equal(gk[order], want[0][worder])
+    assert np.array_equal(gs[order], want[1][worder])
+
+
+N_GB = 1 << 20  # from here on the key order is looked at
+
+
+def runs_of(rng, n, longest):
+    """Ascending keys (with gaps) in runs of 1..longest rows."""
+    m = min(n, 4 * n // (longest + 1) + 64)  # runs enough for n rows
+    reps = rng.integers(1, longest + 1, size=m)
+    reps[-1] += max(0, n - int(reps.sum()))
+    keys = np.cumsum(rng.integers(1, 9, size=m))
+    return np.repeat(keys, reps)[:n].astype(np.int64)
+
+
+@pytest.mark.parametrize("longest", [1, 7, 300, 200_000])
+@pytest.mark.parametrize("n", [N_GB - 1, N_GB, N_GB + 1, 3_000_017])
+@pytest.mark.parametrize("off", [0, 1])
+def test_groupby_in_key_order(ctx, stream, longest, n, off):
+    """Runs that end at, span and cross the shares of the warps."""
+    rng = np.random.default_rng(n + longest)
+    k = runs_of(rng, n, longest) - 1000
+    check_groupby(ctx, stream, k, rng.integers(-10**12, 10**12, size=n), off=off)
+
+
+@pytest.mark.parametrize("kt,vt", [(np.int32, np.int8), (np.int8, np.int32), (np.int32, np.int64)])
+def test_groupby_in_key_order_types(ctx, stream, kt, vt):
+    rng = np.random.default_rng(2)
+    n = N_GB + 777
+    k = np.sort(rng.integers(-100, 100, size=n)).astype(kt) if kt == np.int8 else \
+        runs_of(rng, n, 5).astype(kt)
+    v = rng.integers(np.iinfo(vt).min // 2, np.iinfo(vt).max // 2, size=n).astype(vt)
+    check_groupby(ctx, stream, k, (v >> 20).astype(vt) if vt == np.int64 else v)
+
+
+# A late part after one descent: rows of groups seen before and of new ones.
+@pytest.mark.parametrize("tail", [1, 129, 100_000, 700_000])
+@pytest.mark.parametrize("new", [False, True])
+def test_groupby_with_a_late_part(ctx, stream, tail, new):
+    rng = np.random.default_rng(tail)
+    n = 2 * N_GB
+    k = runs_of(rng, n, 4)
+    k[n - tail:] = np.sort(rng.integers(0, k[n - tail - 1] + (1000 if new else 0), size=tail))
+    k[n - tail] = 0 if new else k[0]  # the descent
+    check_groupby(ctx, stream, k, rng.integers(0, 10**9, size=n))
+
+
+@pytest.mark.parametrize("kind", ["all-equal", "two-descents", "reversed", "zipf", "zipf-sparse",
+                                  "uniform-sparse", "cancelling", "wrapping"])
+def test_groupby_other_orders(ctx, stream, kind):
+    rng = np.random.default_rng(17)
+    n = N_GB + 4321
+    v = rng.integers(-10**9, 10**9, size=n)
+    k = runs_of(rng, n, 4)
+    if kind == "all-equal":
+        k[:] = -5
+    elif kind == "two-descents":
+        k = np.concatenate([k[:n // 3], k[:n // 3], k[:n - 2 * (n // 3)]])
+    elif kind == "reversed":
+        k = k[::-1].copy()
+    elif kind.startswith("zipf"):
+        k = np.exp(rng.random(n) * np.log(200_000)).astype(np.int64) * 7919 % 200_003
+        k = k * 1000 - 10**7 if kind == "zipf-sparse" else k
+    elif kind == "uniform-sparse":
+        k = rng.integers(-2**62, 2**62, size=n // 4)[rng.integers(0, n // 4, size=n)]
+    elif kind == "cancelling":  # sums of exactly 0 are groups too
+        k = np.repeat(np.arange(n // 2 + 1), 2)[:n]
+        v = np.where(np.arange(n) % 2 == 0, 7, -7)
+    elif kind == "wrapping":  # frequent group whose low words carry often
+        k = np.where(rng.random(n) < 0.7, 3, k)
+        v = rng.integers(2**31, 2**40, size=n) * rng.choice([-1, 1], size=n)
+    check_groupby(ctx, stream, k, v)
+
+
+@pytest.mark.parametrize("order", ["runs", "late", "zipf"])
+def test_groupby_capacity_is_counted(ctx, stream, order):
+    rng = np.random.default_rng(3)
+    n = N_GB + 5
+    k = runs_of(rng, n, 4)
+    if order == "late":
+        k[-1000:] = np.arange(1000) * 3
+    elif order == "zipf":
+        k = np.exp(rng.random(n) * np.log(100_000)).astype(np.int64)
+    groups = len(np.unique(k))
+    with torch.cuda.stream(stream):
+        ok, os_, ng = pq.pq_groupby_sum(ctx, dev(k), dev(k), cap=groups - 7, stream=stream)
+        with pytest.raises(pq.PQError) as e:
+            ctx.sync(stream)
+    assert e.value.status == pq.PQ_ERR_CAPACITY and int(ng.item()) == groups
+
+
+def test_groupby_reserved_key_in_order(ctx, stream):
+    k = np.sort(np.random.default_rng(1).integers(-50, 50, size=N_GB))
+    k[0] = np.iinfo(np.int64).min
+    with torch.cuda.stream(stream):
+        ok, os_, ng = pq.pq_groupby_sum(ctx, dev(k), dev(k), cap=1000, stream=stream)
+        with pytest.raises(pq.PQError) as e:
+            ctx.sync(stream)
+    assert e.value.status == pq.PQ_ERR_RESERVED_KEY
+    assert int(ng.item()) == len(np.unique(k)) - 1
+
+
+# Blocks with 8 pairs and more per thread read the sums first.
+@pytest.mark.parametrize("n", [2047, 2048, 2049, 700_001, 2_500_000])
+@pytest.mark.parametrize("kind", ["random", "equal", "few", "ascending"])
+def test_topk_sums_first(ctx, stream, n, kind):
+    rng = np.random.default_rng(n)
+    keys = rng.permutation(n).astype(np.int64) - n // 2
+    sums = {"random": rng.integers(-2**62, 2**62, size=n), "equal": np.full(n, -3),
+            "few": rng.integers(0, 5, size=n), "ascending": np.arange(n) * 3}[kind].astype(np.int64)
+    for k in (1, 10, 32, 33):
+        with torch.cuda.stream(stream):
+            ok, os_, nout = pq.pq_topk(ctx, dev(keys), dev(sums), k, stream=stream)
+            ctx.sync(stream)
+        wk, ws = oracle.topk(keys, sums, k)
+        assert int(nout.item()) == len(wk)
+        assert np.array_equal(ok[:len(wk)].cpu().numpy(), wk)
+        assert np.array_equal(os_[:len(wk)].cpu().numpy(), ws)
