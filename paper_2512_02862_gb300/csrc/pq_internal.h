@@ -193,7 +193,7 @@ struct pq_table {
 struct pq_ht {
   pqk::i64* keys = nullptr;
   pqk::i64* vals = nullptr;  // keys + 1: slots are {key, value} pairs
-  pqk::i64* meta = nullptr;   // [0] duplicate-key flag, [1] inserted count
+  pqk::i64* meta = nullptr;   // HtMeta (pq_ops.cu): duplicate-key flag, key order
   int log2cap = 0;
   int64_t n = 0;
   void* block = nullptr;

@@ -211,3 +211,75 @@ def test_topk_sums_first(ctx, stream, n, kind):
         assert int(nout.item()) == len(wk)
         assert np.array_equal(ok[:len(wk)].cpu().numpy(), wk)
         assert np.array_equal(os_[:len(wk)].cpu().numpy(), ws)
+
+
+N_HT = 1 << 18  # build keys from which lines of the table may follow the key order
+
+
+def join_keys(rng, kind, n):
+    i = np.arange(n, dtype=np.int64)
+    if kind == "gap4":
+        return 4 * i + rng.integers(0, 4, size=n) - 2 * n
+    if kind == "gap1000":
+        return 1000 * i + rng.integers(0, 1000, size=n)
+    if kind == "dense":
+        return i - n // 3
+    if kind == "two-scales":    # regions of dense ids
+        return (i // 500 << 40) + i % 500
+    if kind == "outliers":      # dense ids and a few keys far away
+        k = i.copy()
+        k[::1000] = rng.integers(-2**62, 2**62, size=len(k[::1000]))
+        return k
+    if kind == "half-sparse":   # the sample's spacing fits neither half
+        return np.where(i < n // 2, i, i * 5000)
+    if kind == "random":
+        return rng.integers(-2**62, 2**62, size=n)
+    if kind == "equal-low-bits":
+        return i << 34
+    if kind == "repeated":      # lines fill up with copies of a key
+        return np.repeat(4 * np.arange(n // 5 + 1), 5)[:n]
+    if kind == "few-repeated-much":
+        return np.where(rng.random(n) < 0.001, 4 * 77, 4 * i)
+    raise ValueError(kind)
+
+
+@pytest.mark.parametrize("n", [N_HT - 1, N_HT, N_HT + 12_345])
+@pytest.mark.parametrize("kind", ["gap4", "gap1000", "dense", "two-scales", "outliers",
+                                  "half-sparse", "random", "equal-low-bits", "repeated",
+                                  "few-repeated-much"])
+def test_join_key_order(ctx, stream, n, kind):
+    rng = np.random.default_rng(n)
+    build = join_keys(rng, kind, n)
+    if kind in ("dense", "random"):
+        rng.shuffle(build)
+    vals = rng.integers(-10**12, 10**12, size=n)
+    probe = np.concatenate([build[rng.integers(0, n, size=20_011)],
+                            build[:500] + 1, build[-500:] - 1, np.array([0, 2**62, -2**62])])
+    wr, wv = oracle.join(build, probe, vals)
+    with torch.cuda.stream(stream):
+        ht = pq.pq_join_build(ctx, dev(build), dev(vals), stream=stream)
+        rows, got, cnt = pq.pq_join_probe(ctx, ht, dev(probe), cap=len(wr) + 5, stream=stream)
+        ht.free(stream)
+        ctx.sync(stream)
+    c = int(cnt.item())
+    assert c == len(wr)
+    rows, got = rows[:c].cpu().numpy(), got[:c].cpu().numpy()
+    order, worder = np.lexsort((got, rows)), np.lexsort((wv, wr))
+    assert np.array_equal(rows[order], wr[worder]) and np.array_equal(got[order], wv[worder])
+
+
+def test_join_key_order_int32_row_ids(ctx, stream):
+    rng = np.random.default_rng(4)
+    n = N_HT + 3
+    build = (rng.permutation(n) * 3 - n).astype(np.int32)
+    probe = np.arange(-n, 2 * n, dtype=np.int32)
+    wr, wv = oracle.join(build, probe)
+    with torch.cuda.stream(stream):
+        ht = pq.pq_join_build(ctx, dev(build), None, load_factor=0.9, stream=stream)
+        rows, got, cnt = pq.pq_join_probe(ctx, ht, dev(probe), cap=len(wr), stream=stream)
+        ht.free(stream)
+        ctx.sync(stream)
+    assert int(cnt.item()) == len(wr)
+    order = np.argsort(rows.cpu().numpy())
+    assert np.array_equal(rows.cpu().numpy()[order], wr)
+    assert np.array_equal(got.cpu().numpy()[order], wv)
