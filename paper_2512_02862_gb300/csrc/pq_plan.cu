@@ -826,6 +826,20 @@ pq_status run_batch_internal(pq_ctx* ctx, const pq_plan* plans, int n, pq_result
     off[i] = total;
     total += plan_bytes(R[i]);
   }
+  // Scan tiles sized for the batch: its plans share the grid, so it is the
+  // rows of all of them that have to give every warp two tiles.  (Sized by
+  // each plan's own rows, 64 plans of 1.3M F rows on average were scanned in
+  // 128-row tiles, each with a ticket, a search for its plan and the plan's
+  // constants to load: F scans 562 -> 180 us, M scans 267 -> 113 us.)
+  if (n > 1) {
+    i64 nd = 0, nm = 0, nf = 0;
+    for (const ResolvedPlan& r : R) nd += r.builds ? r.n_d : 0, nm += r.n_m, nf += r.n_f;
+    for (ResolvedPlan& r : R) {
+      r.dev.d_tile = scan_tile(nd, 512, kTD, resident_warps(ctx, 0));
+      r.dev.m_tile = scan_tile(nm, 128, kTM, resident_warps(ctx, 3));
+      r.dev.f_tile = scan_tile(nf, 128, kTF, resident_warps(ctx, 8));
+    }
+  }
   char* ws = (char*)ctx->arena.alloc(total);
   if (!ws) {
     unwind();
