@@ -506,6 +506,22 @@ constexpr int kSub = 2048;
 constexpr int kSubWarpRows = kSub / 8;     // rows of a warp in a sub-tile
 constexpr int kSubSteps = kSubWarpRows / 32;
 
+// The part of the bucket number that a pass orders by: `bits` bits from
+// `shift` on of a number of log2P bits (all of it, or half of it in a partition
+// in two passes).  One multiply, shift and mask per key.
+struct Digit {
+  int log2P, bits, rshift;
+  u32 mask;
+  Digit() = default;
+  __host__ __device__ Digit(int log2P_, int shift, int bits_)
+      : log2P(log2P_), bits(bits_), rshift(log2P_ ? 64 - log2P_ + shift : 63),
+        mask((1u << bits_) - 1u) {}
+  __host__ __device__ int count() const { return 1 << bits; }
+  __device__ __forceinline__ u32 operator()(i64 k) const {
+    return (u32)(((u64)k * 0x9E3779B97F4A7C15ULL) >> rshift) & mask;
+  }
+};
+
 // Lanes of the warp whose bucket equals this lane's, from one ballot per
 // bucket bit (all lanes taking part): cheaper than a general match for small
 // bucket ids.  nbits = log2P when every lane holds a row; otherwise
@@ -534,10 +550,14 @@ __host__ __device__ inline i64 chunk_begin(i64 n, i64 g, i64 k) {
 // its counts into hist[b * g + k] (zeroed before).
 template <typename T>
 __global__ void __launch_bounds__(256, 8) k_part_hist_blk(const T* __restrict__ key, i64 n,
-                                                          int log2P, u32* __restrict__ hist,
-                                                          i64 g, int hsplit) {
+                                                          Digit dg, u32* __restrict__ hist,
+                                                          i64 g, int hsplit,
+                                                          u32* __restrict__ tot) {
   extern __shared__ u32 sh[];
-  const int P = 1 << log2P;
+  // With `tot` (the first of two passes) whole buckets are counted, into tot
+  // and, added up by digit, into hist.
+  const int P = tot ? 1 << dg.log2P : dg.count();
+  const Digit cd = tot ? Digit(dg.log2P, 0, dg.log2P) : dg;
   for (int b = threadIdx.x; b < P; b += blockDim.x) sh[b] = 0;
   __syncthreads();
   const i64 k = blockIdx.x / hsplit, h = blockIdx.x % hsplit;
@@ -563,14 +583,26 @@ __global__ void __launch_bounds__(256, 8) k_part_hist_blk(const T* __restrict__ 
       T v[kPerVec];
       memcpy(v, &x[j], 16);
 #pragma unroll
-      for (int e = 0; e < kPerVec; ++e) atomicAdd(&sh[fib_bucket((i64)v[e], log2P)], 1u);
+      for (int e = 0; e < kPerVec; ++e) atomicAdd(&sh[cd((i64)v[e])], 1u);
     }
   }
   for (i64 i = r0 + steps * kRows + threadIdx.x; i < r1; i += blockDim.x)
-    atomicAdd(&sh[fib_bucket((i64)__ldg(key + i), log2P)], 1u);
+    atomicAdd(&sh[cd((i64)__ldg(key + i))], 1u);
   __syncthreads();
+  if (!tot) {
+    for (int b = threadIdx.x; b < P; b += blockDim.x)
+      if (sh[b]) atomicAdd(&hist[(i64)b * g + k], sh[b]);
+    return;
+  }
   for (int b = threadIdx.x; b < P; b += blockDim.x)
-    if (sh[b]) atomicAdd(&hist[(i64)b * g + k], sh[b]);
+    if (sh[b]) atomicAdd(&tot[b], sh[b]);
+  // Lane l of a warp adds up a digit's buckets l, l + 32, ...
+  for (int d = warp; d < dg.count(); d += 8) {
+    u32 c = 0;
+    for (int o = lane; o < P >> dg.bits; o += 32) c += sh[(o << dg.bits) | d];  // shift 0
+    c = __reduce_add_sync(kFull, c);
+    if (lane == 0 && c) atomicAdd(&hist[(i64)d * g + k], c);
+  }
 }
 
 // Shared memory of the staged scatter for P buckets (bytes).
@@ -618,11 +650,11 @@ __device__ __forceinline__ void stage_column(const V* __restrict__ src, V* __res
 
 template <typename T>
 __global__ void __launch_bounds__(256) k_part_scatter_blk(const T* __restrict__ key, i64 n,
-                                                          int log2P, const i64* __restrict__ gofs,
+                                                          Digit dg, const i64* __restrict__ gofs,
                                                           PayArgs pa, T* __restrict__ out_key,
                                                           i64* d_offsets) {
   extern __shared__ __align__(16) unsigned char smem[];
-  const int P = 1 << log2P;
+  const int log2P = dg.bits, P = 1 << log2P;
   i64* s_gb = reinterpret_cast<i64*>(smem);
   u32* s_cnt = reinterpret_cast<u32*>(s_gb + P);
   u32* s_run = s_cnt + 8 * P;
@@ -635,9 +667,9 @@ __global__ void __launch_bounds__(256) k_part_scatter_blk(const T* __restrict__ 
   const i64 r0 = chunk_begin(n, g, k), r1 = chunk_begin(n, g, k + 1);
   for (int b = threadIdx.x; b < P; b += blockDim.x) {
     s_gb[b] = gofs[(i64)b * g + k];
-    if (k == 0) d_offsets[b] = s_gb[b];
+    if (k == 0 && d_offsets) d_offsets[b] = s_gb[b];
   }
-  if (k == 0 && threadIdx.x == 0) d_offsets[P] = n;
+  if (k == 0 && threadIdx.x == 0 && d_offsets) d_offsets[P] = n;
   for (i64 r = r0; r < r1; r += kSub) {
     const int cnt = (int)min((i64)kSub, r1 - r);
     for (int b = threadIdx.x; b < 8 * P; b += blockDim.x) s_cnt[b] = 0;
@@ -649,7 +681,7 @@ __global__ void __launch_bounds__(256) k_part_scatter_blk(const T* __restrict__ 
 #pragma unroll
     for (int st = 0; st < kSubSteps; ++st) {
       const int i = warp * kSubWarpRows + st * 32 + lane;
-      bp[st] = i < cnt ? fib_bucket((i64)__ldg(key + r + i), log2P) : 0xFFFFFFFFu;
+      bp[st] = i < cnt ? dg((i64)__ldg(key + r + i)) : 0xFFFFFFFFu;
     }
 #pragma unroll
     for (int st = 0; st < kSubSteps; ++st) {
@@ -765,8 +797,10 @@ __device__ __forceinline__ void gather_column(const char* buf, int off, V* __res
     if (j * 256 + (int)threadIdx.x < cnt) __stcs(dst + drow[j], col[src[j]]);
 }
 
+// (Three blocks per SM, as the buffers allow: left alone, the compiler holds it
+// to 40 registers with a spill, 5 % slower in two passes.)
 template <typename T, int SUB>
-__global__ void __launch_bounds__(256) k_part_scatter_tma(i64 n, int log2P,
+__global__ void __launch_bounds__(256, 3) k_part_scatter_tma(i64 n, Digit dg,
                                                           const i64* __restrict__ gofs,
                                                           TmaCols tc, i64* d_offsets,
                                                           i64 spin_limit, DevStatus* st) {
@@ -774,7 +808,7 @@ __global__ void __launch_bounds__(256) k_part_scatter_tma(i64 n, int log2P,
   constexpr int kSteps = kWRows / 32;
   static_assert(kWRows <= 512, "place takes 9 bits");
   extern __shared__ __align__(16) unsigned char smem[];
-  const int P = 1 << log2P;
+  const int log2P = dg.bits, P = 1 << log2P;
   u64* bar = reinterpret_cast<u64*>(smem);
   char* bufs = reinterpret_cast<char*>(smem + 16);
   i64* s_gb = reinterpret_cast<i64*>(bufs + 2 * (size_t)tc.buf_bytes);
@@ -794,9 +828,9 @@ __global__ void __launch_bounds__(256) k_part_scatter_tma(i64 n, int log2P,
   }
   for (int b = threadIdx.x; b < P; b += blockDim.x) {
     s_gb[b] = gofs[(i64)b * g + k];
-    if (k == 0) d_offsets[b] = s_gb[b];
+    if (k == 0 && d_offsets) d_offsets[b] = s_gb[b];
   }
-  if (k == 0 && threadIdx.x == 0) d_offsets[P] = n;
+  if (k == 0 && threadIdx.x == 0 && d_offsets) d_offsets[P] = n;
   __syncthreads();
   // Thread 0 starts the copies of sub-tile j into buffer j & 1: the part of
   // each column slice that is a whole number of 16-byte units (all of it but
@@ -851,7 +885,7 @@ __global__ void __launch_bounds__(256) k_part_scatter_tma(i64 n, int log2P,
 #pragma unroll
     for (int q = 0; q < kSteps; ++q) {
       const int i = warp * kWRows + q * 32 + lane;
-      bp[q] = i < cnt ? fib_bucket((i64)s_key[i], log2P) : 0xFFFFFFFFu;
+      bp[q] = i < cnt ? dg((i64)s_key[i]) : 0xFFFFFFFFu;
     }
 #pragma unroll
     for (int q = 0; q < kSteps; ++q) {
@@ -1936,6 +1970,139 @@ pq_status pq_filter(pq_ctx* ctx, pq_col col, int op, int64_t c, const int64_t* s
   return PQ_OK;
 }
 
+}  // extern "C"
+
+namespace {
+// Blocks of a scatter kernel resident per SM with `smem` bytes of dynamic
+// shared memory; what does not depend on smem is asked of the runtime once.
+template <auto K>
+int part_blocks(size_t smem) {
+  static const int most = [] {
+    int occ = 0;
+    if (cudaFuncSetAttribute((const void*)K, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             200 * 1024) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, (const void*)K, 256, 0) != cudaSuccess)
+      cudaGetLastError();
+    return std::max(occ, 1);
+  }();
+  constexpr size_t kPerSm = 228 * 1024, kPerBlock = 1024 + 256;  // reserved and static, per block
+  return std::max(1, std::min(most, (int)(kPerSm / (smem + kPerBlock))));
+}
+
+// One stable pass of the partition: rows ordered by digit `dg` of their
+// bucket.  d_offsets: the digits' offsets (or null); tot: null, or counts of
+// whole buckets to be added to (zeroed by the caller).
+pq_status part_pass(pq_ctx* ctx, pq_col key, const pq_col* payload, int npay, Digit dg,
+                    void* out_key, void* const* out_payload, i64* d_offsets, u32* tot,
+                    cudaStream_t s) {
+  const i64 n = key.n;
+  const int P = dg.count();
+  PayArgs pa{};
+  pa.n = npay;
+  for (int j = 0; j < npay; ++j) {
+    pa.src[j] = payload[j].data;
+    pa.dst[j] = out_payload[j];
+    pa.type[j] = payload[j].type;
+  }
+  // Staged scatter: G persistent blocks, one chunk of rows each; with bulk
+  // copies into double-buffered sub-tiles when every column is 16-byte
+  // aligned and the buffers fit.
+  TmaCols tc{};
+  tc.n = 1 + npay;
+  tc.src[0] = key.data;
+  tc.dst[0] = out_key;
+  tc.es[0] = (int)pqh::dtype_size(key.type);
+  bool aligned = ((uintptr_t)key.data & 15) == 0 && ((uintptr_t)out_key & 15) == 0;
+  for (int j = 0; j < npay; ++j) {
+    tc.src[1 + j] = payload[j].data;
+    tc.dst[1 + j] = out_payload[j];
+    tc.es[1 + j] = (int)pqh::dtype_size(payload[j].type);
+    aligned = aligned && ((uintptr_t)payload[j].data & 15) == 0;
+  }
+  // Sub-tiles of 4096 rows from 512 buckets on (when they fit; of narrow rows
+  // from 256 on), so that a bucket's run in a sub-tile fills its sectors; 2048
+  // otherwise.
+  auto layout = [&](int sub) {
+    int off = 0;
+    for (int c = 0; c < tc.n; ++c) tc.off[c] = off, off += sub * tc.es[c];
+    tc.buf_bytes = off;
+    return tma_smem(P, tc.buf_bytes, sub);
+  };
+  int sub = 4096;
+  size_t smem_tma = layout(sub);
+  if (dg.bits < 8 || (dg.bits == 8 && tc.buf_bytes > 32 * 1024) || smem_tma > 200 * 1024)
+    smem_tma = layout(sub = kSub);
+  const bool use_tma = aligned && smem_tma <= 200 * 1024;
+  const size_t smem = use_tma ? smem_tma : staged_smem(P);
+  const i64 rows_sub = use_tma ? sub : kSub;
+  int occ = 1;
+  PQ_DISPATCH_T(key.type, T, {
+    occ = !use_tma      ? part_blocks<k_part_scatter_blk<T>>(smem)
+          : sub == 4096 ? part_blocks<k_part_scatter_tma<T, 4096>>(smem)
+                        : part_blocks<k_part_scatter_tma<T, kSub>>(smem);
+  });
+  const i64 g = std::max<i64>(1, std::min<i64>((n + rows_sub - 1) / rows_sub,
+                                               (i64)ctx->num_sms * occ));
+  const i64 m = g * P;
+  const i64 stiles = (m + 4095) / 4096;
+  // One block of scratch: the scan's state and the histogram (both zeroed),
+  // then the scanned offsets.
+  pqh::Scratch scr(ctx, s);
+  const size_t w_b = (size_t)(stiles * 8 + 256 + 255) / 256 * 256;
+  const size_t hist_b = (size_t)(m * 4 + 255) / 256 * 256;
+  char* w = (char*)scr.get(w_b + hist_b + m * 8);
+  if (!w) return pqh::fail(ctx, PQ_ERR_BUDGET, "pq_partition: no scratch");
+  u32* hist = (u32*)(w + w_b);
+  i64* gofs = (i64*)(w + w_b + hist_b);
+  PQ_CUDA(ctx, cudaMemsetAsync(w, 0, w_b + hist_b, s));
+  // Histogram blocks: at most one wave of eight per SM (hsplit blocks per
+  // chunk), each with at least 4096 rows; one per chunk where whole buckets
+  // are counted, so that fewer blocks add their counts of up to 4096 buckets.
+  const int hsplit = tot ? 1 : (int)std::max<i64>(
+      1, std::min<i64>(((i64)ctx->num_sms * 8) / g, (n / g) / 4096));
+  PQ_DISPATCH_T(key.type, T, {
+    k_part_hist_blk<T><<<(unsigned)(g * hsplit), 256, (size_t)(tot ? 1 << dg.log2P : P) * 4, s>>>(
+        (const T*)key.data, n, dg, hist, g, hsplit, tot);
+    PQ_LAUNCHED(ctx);
+    k_scan_u32<<<(unsigned)std::min<i64>(stiles, (i64)ctx->num_sms * 4), 256, 0, s>>>(
+        hist, m, gofs, (u64*)(w + 256), (u32*)w, ctx->opt.spin_limit, ctx->d_status);
+    PQ_LAUNCHED(ctx);
+    auto tma = [&](auto k) {
+      k<<<(unsigned)g, 256, smem, s>>>(n, dg, gofs, tc, d_offsets, ctx->opt.spin_limit,
+                                       ctx->d_status);
+    };
+    if (!use_tma)
+      k_part_scatter_blk<T><<<(unsigned)g, 256, smem, s>>>((const T*)key.data, n, dg, gofs, pa,
+                                                           (T*)out_key, d_offsets);
+    else if (sub == 4096)
+      tma(k_part_scatter_tma<T, 4096>);
+    else
+      tma(k_part_scatter_tma<T, kSub>);
+  });
+  PQ_LAUNCHED(ctx);
+  return PQ_OK;
+}
+
+// Whether a partition takes two passes: each writes runs of 64 and more rows
+// per bucket and sub-tile, where one pass by 1024 buckets writes runs of two
+// to four (partly written sectors, and 8 x 1024 counters a sub-tile that leave
+// room for one block per SM), and above that 8192-row tiles are scattered row
+// by row.  It moves the rows twice and takes nine more launches, so it pays
+// from some size on.  20M rows of 21 bytes by 1024: 0.67 -> 0.46 ms, 60M of
+// 16 bytes 1.10 -> 1.02 ms (20M of them 0.41 either way; by 512 buckets one
+// pass is faster, 0.98 against 0.99 ms); 20M rows of 16 bytes by 2048 0.65 -> 0.42 ms, by
+// 4096 1.33 -> 0.43 ms; 4M of them by 2048 0.18 -> 0.17 ms, by 4096 0.31 -> 0.17.
+bool part_two_passes(int log2P, i64 n, const pq_col& key, const pq_col* payload, int npay) {
+  i64 row = (i64)pqh::dtype_size(key.type);
+  for (int j = 0; j < npay; ++j) row += (i64)pqh::dtype_size(payload[j].type);
+  const i64 bytes = n * row;
+  return bytes >= (log2P == 10 ? 320LL << 20 : log2P == 11 ? 48LL << 20 : 16LL << 20) &&
+         log2P >= 10;
+}
+}  // namespace
+
+extern "C" {
+
 pq_status pq_partition(pq_ctx* ctx, pq_col key, const pq_col* payload, int npay, int log2P,
                        void* out_key, void* const* out_payload, int64_t* d_offsets,
                        void* stream) {
@@ -1962,81 +2129,48 @@ pq_status pq_partition(pq_ctx* ctx, pq_col key, const pq_col* payload, int npay,
     return PQ_OK;
   }
   if (!key.data || !out_key) return pqh::fail(ctx, PQ_ERR_INVALID_ARG, "pq_partition: null key");
-  if (log2P <= kStagedMaxLog2) {
-    // Staged scatter: G persistent blocks, one chunk of rows each; with bulk
-    // copies into double-buffered sub-tiles when every column is 16-byte
-    // aligned and the buffers fit.
-    TmaCols tc{};
-    tc.n = 1 + npay;
-    tc.src[0] = key.data;
-    tc.dst[0] = out_key;
-    tc.es[0] = (int)pqh::dtype_size(key.type);
-    bool aligned = ((uintptr_t)key.data & 15) == 0 && ((uintptr_t)out_key & 15) == 0;
-    for (int j = 0; j < npay; ++j) {
-      tc.src[1 + j] = payload[j].data;
-      tc.dst[1 + j] = out_payload[j];
-      tc.es[1 + j] = (int)pqh::dtype_size(payload[j].type);
-      aligned = aligned && ((uintptr_t)payload[j].data & 15) == 0;
-    }
-    // Sub-tiles of 4096 rows from 512 buckets on (when they fit), so that a
-    // bucket's run in a sub-tile fills its sectors; 2048 otherwise.
-    auto layout = [&](int sub) {
-      int off = 0;
-      for (int c = 0; c < tc.n; ++c) tc.off[c] = off, off += sub * tc.es[c];
-      tc.buf_bytes = off;
-      return tma_smem(P, tc.buf_bytes, sub);
-    };
-    int sub = log2P >= 9 ? 4096 : kSub;
-    size_t smem_tma = layout(sub);
-    if (smem_tma > 200 * 1024 && sub != kSub) smem_tma = layout(sub = kSub);
-    const bool use_tma = aligned && smem_tma <= 200 * 1024;
-    const size_t smem = use_tma ? smem_tma : staged_smem(P);
-    const i64 rows_sub = use_tma ? sub : kSub;
-    int occ = 1;
-    PQ_DISPATCH_T(key.type, T, {
-      const void* fn = !use_tma      ? (const void*)k_part_scatter_blk<T>
-                       : sub == 4096 ? (const void*)k_part_scatter_tma<T, 4096>
-                                     : (const void*)k_part_scatter_tma<T, kSub>;
-      cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, 256, smem) != cudaSuccess)
-        occ = 1;
-    });
-    cudaGetLastError();
-    const i64 g = std::max<i64>(1, std::min<i64>((n + rows_sub - 1) / rows_sub,
-                                                 (i64)ctx->num_sms * std::max(occ, 1)));
-    const i64 m = g * P;
-    const i64 stiles = (m + 4095) / 4096;
+  // Many buckets: two stable passes, by the low half of the bucket number into
+  // scratch and by the high half into the output, when the scratch fits.
+  if (part_two_passes(log2P, n, key, payload, npay)) {
     pqh::Scratch scr(ctx, s);
-    u32* hist = (u32*)scr.get(m * 4);
-    i64* gofs = (i64*)scr.get(m * 8);
-    char* w = (char*)scr.get(stiles * 8 + 256);
-    if (!hist || !gofs || !w) return pqh::fail(ctx, PQ_ERR_BUDGET, "pq_partition: no scratch");
-    PQ_CUDA(ctx, cudaMemsetAsync(w, 0, stiles * 8 + 256, s));
-    PQ_CUDA(ctx, cudaMemsetAsync(hist, 0, m * 4, s));
-    // Histogram blocks: at most one wave of eight per SM (hsplit blocks per
-    // chunk), each with at least 4096 rows.
-    const int hsplit = (int)std::max<i64>(
-        1, std::min<i64>(((i64)ctx->num_sms * 8) / g, (n / g) / 4096));
-    PQ_DISPATCH_T(key.type, T, {
-      k_part_hist_blk<T><<<(unsigned)(g * hsplit), 256, (size_t)P * 4, s>>>(
-          (const T*)key.data, n, log2P, hist, g, hsplit);
-      PQ_LAUNCHED(ctx);
-      k_scan_u32<<<(unsigned)std::min<i64>(stiles, (i64)ctx->num_sms * 4), 256, 0, s>>>(
-          hist, m, gofs, (u64*)(w + 256), (u32*)w, ctx->opt.spin_limit, ctx->d_status);
-      PQ_LAUNCHED(ctx);
-      if (use_tma && sub == 4096)
-        k_part_scatter_tma<T, 4096><<<(unsigned)g, 256, smem, s>>>(
-            n, log2P, gofs, tc, (i64*)d_offsets, ctx->opt.spin_limit, ctx->d_status);
-      else if (use_tma)
-        k_part_scatter_tma<T, kSub><<<(unsigned)g, 256, smem, s>>>(
-            n, log2P, gofs, tc, (i64*)d_offsets, ctx->opt.spin_limit, ctx->d_status);
-      else
-        k_part_scatter_blk<T><<<(unsigned)g, 256, smem, s>>>((const T*)key.data, n, log2P, gofs,
-                                                             pa, (T*)out_key, (i64*)d_offsets);
-    });
-    PQ_LAUNCHED(ctx);
-    return PQ_OK;
+    size_t bytes = 0;
+    auto put = [&](int type) {
+      const size_t at = bytes;
+      bytes += ((size_t)n * pqh::dtype_size(type) + 255) / 256 * 256;
+      return at;
+    };
+    size_t at[1 + PQ_MAX_PAYLOAD];
+    at[0] = put(key.type);
+    for (int j = 0; j < npay; ++j) at[1 + j] = put(payload[j].type);
+    char* w = (char*)scr.get(bytes);
+    const size_t tot_b = (size_t)P * 4;
+    char* t = w ? (char*)scr.get(512 + tot_b) : nullptr;
+    if (t) {
+      u32* tot = (u32*)(t + 512);
+      PQ_CUDA(ctx, cudaMemsetAsync(t, 0, 512 + tot_b, s));
+      const int lo = log2P / 2;
+      pq_col k1 = key, p1[PQ_MAX_PAYLOAD];
+      void* o1[PQ_MAX_PAYLOAD];
+      k1.data = w + at[0];
+      for (int j = 0; j < npay; ++j) p1[j] = payload[j], p1[j].data = o1[j] = w + at[1 + j];
+      pq_status st = part_pass(ctx, key, payload, npay, Digit(log2P, 0, lo), w + at[0], o1, nullptr,
+                               tot, s);
+      if (st == PQ_OK)
+        st = part_pass(ctx, k1, p1, npay, Digit(log2P, lo, log2P - lo), out_key, out_payload,
+                       nullptr, nullptr, s);
+      if (st == PQ_OK) {
+        // The buckets' offsets from their counts (P <= 4096: one tile).
+        k_scan_u32<<<1, 256, 0, s>>>(tot, P, (i64*)d_offsets, (u64*)(t + 256), (u32*)t,
+                                     ctx->opt.spin_limit, ctx->d_status);
+        PQ_LAUNCHED(ctx);
+        return pqh::fill_i64(ctx, (i64*)d_offsets + P, 1, n, s);
+      }
+      if (st != PQ_ERR_BUDGET) return st;
+    }
   }
+  if (log2P <= kStagedMaxLog2)
+    return part_pass(ctx, key, payload, npay, Digit(log2P, 0, log2P), out_key, out_payload,
+                     (i64*)d_offsets, nullptr, s);
   const i64 ntiles = (n + kPartTile - 1) / kPartTile;
   const i64 m = ntiles * P;
   const i64 stiles = (m + 4095) / 4096;

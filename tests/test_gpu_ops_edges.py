@@ -283,3 +283,51 @@ def test_join_key_order_int32_row_ids(ctx, stream):
     order = np.argsort(rows.cpu().numpy())
     assert np.array_equal(rows.cpu().numpy()[order], wr)
     assert np.array_equal(got.cpu().numpy()[order], wv)
+
+
+def check_partition(ctx, stream, key, pays, log2P, off=0):
+    want_k, want_p, want_o = oracle.partition(key[off:], log2P, [p[off:] for p in pays])
+    k, ps = dev(key)[off:], [dev(p)[off:] for p in pays]
+    torch.cuda.synchronize()
+    with torch.cuda.stream(stream):
+        gk, gp, go = pq.pq_partition(ctx, k, ps, log2P=log2P, stream=stream)
+        ctx.sync(stream)
+    assert np.array_equal(go.cpu().numpy(), want_o)
+    assert np.array_equal(gk.cpu().numpy(), want_k)
+    for g, w in zip(gp, want_p):
+        assert np.array_equal(g.cpu().numpy(), w)
+
+
+def rows_for(rng, n, kt, pay, dist):
+    hi = 2**31 - 1 if kt == np.int32 else 2**62
+    key = rng.integers(-hi, hi, size=n) if dist == "uniform" else \
+        np.where(rng.random(n) < 0.8, 12345, rng.integers(0, 5000, size=n))
+    return key.astype(kt), [rng.integers(-100, 100, size=n).astype(t) for t in pay]
+
+
+# Two passes by half the bucket number each: 1024 buckets from 320 MiB on,
+# 2048 from 48 MiB, 4096 from 16 MiB; one pass below.
+@pytest.mark.parametrize("log2P,n,kt,pay", [
+    (10, 16_000_001, np.int64, (np.int64, np.int8, np.int32)),
+    (10, 1_000_003, np.int64, (np.int64, np.int8, np.int32)),
+    (11, 6_291_455, np.int32, (np.int32,)), (11, 6_291_456, np.int32, (np.int32,)),
+    (12, 2_097_151, np.int64, ()), (12, 2_097_152, np.int64, ()),
+    (12, 1_300_001, np.int64, (np.int8, np.int32, np.int8)),
+    (8, 1_000_003, np.int32, (np.int32,)), (8, 1_000_003, np.int64, (np.int8,))])
+@pytest.mark.parametrize("dist", ["uniform", "skewed"])
+def test_partition_passes(ctx, stream, log2P, n, kt, pay, dist):
+    check_partition(ctx, stream, *rows_for(np.random.default_rng(n), n, kt, pay, dist), log2P)
+
+
+@pytest.mark.parametrize("log2P", [11, 12])
+def test_partition_two_passes_unaligned(ctx, stream, log2P):
+    key, pays = rows_for(np.random.default_rng(2), 5_000_001, np.int64, (np.int32, np.int8), "uniform")
+    check_partition(ctx, stream, key, pays, log2P, off=1)
+
+
+def test_partition_without_room_for_a_second_copy(stream):
+    """40 MB of rows by 4096 buckets; the arena holds the counts, not the rows."""
+    small = pq.Context(arena_bytes=32 << 20)
+    key, pays = rows_for(np.random.default_rng(3), 2_500_000, np.int64, (np.int64,), "uniform")
+    check_partition(small, stream, key, pays, 12)
+    small.close()
