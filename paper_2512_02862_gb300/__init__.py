@@ -164,20 +164,30 @@ class PQError(RuntimeError):
 
 
 # --------------------------------------------------------------- helpers ----
+_torch_module = None
+_codes: dict = {}   # torch dtype -> pq_dtype
+
+
 def _torch():
-    import torch
-    return torch
+    global _torch_module
+    if _torch_module is None:
+        import torch
+        _codes.update({torch.int8: PQ_INT8, torch.int32: PQ_INT32, torch.int64: PQ_INT64})
+        _torch_module = torch
+    return _torch_module
 
 
 def _dtype_code(t) -> int:
-    torch = _torch()
-    return {torch.int8: PQ_INT8, torch.int32: PQ_INT32, torch.int64: PQ_INT64}[t.dtype]
+    if not _codes:
+        _torch()
+    return _codes[t.dtype]
 
 
 def col(t) -> pq_col:
     """pq_col view of a 1-D contiguous int8/int32/int64 CUDA tensor."""
     assert t.is_cuda and t.dim() == 1 and t.is_contiguous(), "columns are 1-D contiguous CUDA"
-    return pq_col(t.data_ptr() if t.numel() else None, t.numel(), _dtype_code(t), 0)
+    n = t.numel()
+    return pq_col(t.data_ptr() if n else None, n, _dtype_code(t), 0)
 
 
 def _ptr(t):
@@ -185,9 +195,8 @@ def _ptr(t):
 
 
 def _stream(stream):
-    torch = _torch()
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return c_void_p(s.cuda_stream)
+    s = stream if stream is not None else _torch().cuda.current_stream()
+    return s.cuda_stream
 
 
 # Arenas of contexts that pq_destroy could not release (kept until exit).
