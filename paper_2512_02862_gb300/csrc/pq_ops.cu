@@ -1653,9 +1653,10 @@ __global__ void __launch_bounds__(256, 2) k_topk(const i64* __restrict__ keys,
   __shared__ LaneRankSmem<256> s_lr;
   chain_begin();
   const i64 n = d_n ? min(*d_n, n_cap) : n_cap;
-  // Only the first nb blocks take pairs (at least 256 each: one per thread),
-  // so that a small count read on the device leaves few lists to merge.
-  const int nb = (int)max((i64)1, min((i64)gridDim.x, (n + 255) / 256));
+  // Only the first nb blocks take pairs (at least 2048 each: eight per thread),
+  // so that a small count read on the device leaves few lists to merge, or
+  // none.
+  const int nb = (int)max((i64)1, min((i64)gridDim.x, (n + 2047) / 2048));
   if ((int)blockIdx.x >= nb) return;  // no pairs: the nb blocks take the ticket
   const i64 per = (n + nb - 1) / nb;
   const i64 lo = min(n, per * blockIdx.x), hi = min(n, lo + per);

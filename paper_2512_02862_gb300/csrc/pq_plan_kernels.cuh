@@ -181,9 +181,11 @@ __host__ __device__ __forceinline__ DenseLayout dense_layout(i64 c, u64 bits) {
 // Top-k tiling over a first-hit bitmap of `words` words (the hash table's
 // slots, or the dense dictionary's slots).
 __host__ __device__ __forceinline__ i64 topk_tile_words_w(i64 words) {
+  // At most kTKP tiles, as near to it as tiles of 128 words allow (a power of
+  // two left 153 of 256 blocks at 1.25M words).
   i64 tw = 32;
-  while ((words + tw - 1) / tw > kTKP) tw <<= 1;  // at most kTKP tiles
-  return tw;
+  while (tw < 128 && (words + tw - 1) / tw > kTKP) tw <<= 1;
+  return (words + tw - 1) / tw <= kTKP ? tw : (words + kTKP * 128 - 1) / (kTKP * 128) * 128;
 }
 
 __device__ __forceinline__ bool bit_test(const u32* bm, u64 idx, u64 keep) {
