@@ -1,6 +1,7 @@
 // pq_ops.cu -- standalone operators: filter, radix partition, hash-join
 // build/probe, group-by SUM, top-k.
 #include <algorithm>
+#include <atomic>
 #include <cstring>
 #include <mutex>
 
@@ -1012,7 +1013,9 @@ __device__ __forceinline__ u64 ht_slot(const HtPath& p, i64 k, u64 i, u64 mask) 
 // 512 build keys spread over the input (the first and the last among them):
 // their range, and whether each 512th of it holds about one of them.  Keys in
 // no order fail that (random counts reach 4 and more) and gain nothing from
-// it.  One block.
+// it.  Then 512 neighbouring rows at a third and at two thirds of the input:
+// no line gets more of them than it has slots (keys that come in dense groups
+// with gaps between them are hashed).  One block.
 constexpr int kHtSample = 512;
 constexpr i64 kHtSpreadMin = 1 << 18;  // fewer keys: the table lies in L2 whatever the order
 template <typename TK>
@@ -1036,9 +1039,24 @@ __global__ void __launch_bounds__(kHtSample) k_ht_spread(const TK* __restrict__ 
   };
   const bool fits = range >= 8 * lines;  // a slot for one distance or more
   if (fits) atomicAdd(&s_cnt[__umul64hi(u - lo, per_key(kHtSample))], 1u);
-  const int crowded = __syncthreads_or(fits && s_cnt[threadIdx.x] > 3);
+  int crowded = __syncthreads_or(fits && s_cnt[threadIdx.x] > 3);
+  const u64 scale = per_key(8 * lines);
+  for (int h = 1; h <= 2; ++h) {
+    const i64 r0 = n / 3 * h;  // r0 + 511 < n: 2^18 rows at least
+    auto line = [&](i64 r) {
+      const u64 d = ((u64)(i64)__ldg(key + r) ^ 0x8000000000000000ULL) - lo;
+      return __umul64hi(min(d, range), scale) >> 3;
+    };
+    s_cnt[threadIdx.x] = 0;
+    __syncthreads();
+    // Neighbours in key order fall on neighbouring lines: counted modulo 512.
+    const u64 l = fits ? line(r0 + threadIdx.x) : 0;
+    if (fits) atomicAdd(&s_cnt[l % kHtSample], 1u);
+    __syncthreads();
+    crowded |= __syncthreads_or(fits && s_cnt[threadIdx.x] > 8);
+  }
   if (threadIdx.x == 0 && fits && !crowded)
-    meta->umin = lo, meta->range = range, meta->scale = per_key(8 * lines);
+    meta->umin = lo, meta->range = range, meta->scale = scale;
 }
 
 // 15M keys 4i + U{0..3} in order: 0.94 ms when each was hashed by itself (a
@@ -1095,8 +1113,10 @@ __global__ void __launch_bounds__(256) k_ht_build(const TK* __restrict__ key, co
 // wave.  60M rows in key order against 15M build keys: 0.89 ms with each key
 // hashed by itself, 0.50 ms with lines in key order (2 rows per lane: 0.55 ms).
 constexpr int kPrbBuf = 256;
-constexpr int kPrbRows = 4;  // rows per lane in a round
-template <typename TK>
+// ROWS: rows per lane in a round, 4 where every resident warp has several
+// rounds to do; 2 for fewer rows, which more warps then share (a join of 0.9M
+// probes with 225k keys: 182 us a call with 4, 164 with 2).
+template <typename TK, int ROWS>
 __global__ void __launch_bounds__(256, 4) k_ht_probe(const TK* __restrict__ pkey, i64 n,
                                                   const longlong2* __restrict__ slots, int log2cap,
                                                   const HtMeta* meta,
@@ -1125,12 +1145,12 @@ __global__ void __launch_bounds__(256, 4) k_ht_probe(const TK* __restrict__ pkey
   };
   const i64 gw = ((i64)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const i64 nwarps = ((i64)gridDim.x * blockDim.x) >> 5;
-  for (i64 wb = gw * (32 * kPrbRows); wb < n; wb += nwarps * (32 * kPrbRows)) {
-    i64 i[kPrbRows], k[kPrbRows];
-    bool active[kPrbRows];
-    HtPath p[kPrbRows];
+  for (i64 wb = gw * (32 * ROWS); wb < n; wb += nwarps * (32 * ROWS)) {
+    i64 i[ROWS], k[ROWS];
+    bool active[ROWS];
+    HtPath p[ROWS];
 #pragma unroll
-    for (int h = 0; h < kPrbRows; ++h) {
+    for (int h = 0; h < ROWS; ++h) {
       i[h] = wb + h * 32 + lane;
       active[h] = i[h] < n;
       k[h] = active[h] ? (i64)__ldg(pkey + i[h]) : 0;
@@ -1140,14 +1160,14 @@ __global__ void __launch_bounds__(256, 4) k_ht_probe(const TK* __restrict__ pkey
     for (u64 j = 0; j <= mask + 8; ++j) {  // (a table with no free slot: the path ends)
       bool any = false;
 #pragma unroll
-      for (int h = 0; h < kPrbRows; ++h) any |= active[h];
+      for (int h = 0; h < ROWS; ++h) any |= active[h];
       if (!__any_sync(kFull, any)) break;
-      longlong2 kv[kPrbRows];  // {key, value} of each row's current slot
+      longlong2 kv[ROWS];  // {key, value} of each row's current slot
 #pragma unroll
-      for (int h = 0; h < kPrbRows; ++h)
+      for (int h = 0; h < ROWS; ++h)
         kv[h] = active[h] ? __ldg(slots + ht_slot(p[h], k[h], j, mask)) : make_longlong2(kEmpty, 0);
 #pragma unroll
-      for (int h = 0; h < kPrbRows; ++h) {
+      for (int h = 0; h < ROWS; ++h) {
         bool emit = false;
         if (active[h]) {
           if (kv[h].x == kEmpty) {
@@ -1165,7 +1185,7 @@ __global__ void __launch_bounds__(256, 4) k_ht_probe(const TK* __restrict__ pkey
         }
         nb += __popc(em);
       }
-      if (nb > kPrbBuf - 32 * kPrbRows) flush();  // room for a full round stays
+      if (nb > kPrbBuf - 32 * ROWS) flush();  // room for a full round stays
     }
   }
   if (nb) flush();
@@ -1975,17 +1995,21 @@ pq_status pq_filter(pq_ctx* ctx, pq_col col, int op, int64_t c, const int64_t* s
 
 namespace {
 // Blocks of a scatter kernel resident per SM with `smem` bytes of dynamic
-// shared memory; what does not depend on smem is asked of the runtime once.
+// shared memory; what does not depend on smem is asked of the runtime once per
+// device (two threads that ask at once find the same).
 template <auto K>
-int part_blocks(size_t smem) {
-  static const int most = [] {
-    int occ = 0;
+int part_blocks(int device, size_t smem) {
+  static std::atomic<int> known[64];
+  std::atomic<int>* const at = device >= 0 && device < 64 ? &known[device] : nullptr;
+  int most = at ? at->load(std::memory_order_acquire) : 0;
+  if (!most) {
     if (cudaFuncSetAttribute((const void*)K, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              200 * 1024) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, (const void*)K, 256, 0) != cudaSuccess)
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&most, (const void*)K, 256, 0) != cudaSuccess)
       cudaGetLastError();
-    return std::max(occ, 1);
-  }();
+    most = std::max(most, 1);
+    if (at) at->store(most, std::memory_order_release);
+  }
   constexpr size_t kPerSm = 228 * 1024, kPerBlock = 1024 + 256;  // reserved and static, per block
   return std::max(1, std::min(most, (int)(kPerSm / (smem + kPerBlock))));
 }
@@ -2038,9 +2062,9 @@ pq_status part_pass(pq_ctx* ctx, pq_col key, const pq_col* payload, int npay, Di
   const i64 rows_sub = use_tma ? sub : kSub;
   int occ = 1;
   PQ_DISPATCH_T(key.type, T, {
-    occ = !use_tma      ? part_blocks<k_part_scatter_blk<T>>(smem)
-          : sub == 4096 ? part_blocks<k_part_scatter_tma<T, 4096>>(smem)
-                        : part_blocks<k_part_scatter_tma<T, kSub>>(smem);
+    occ = !use_tma      ? part_blocks<k_part_scatter_blk<T>>(ctx->device, smem)
+          : sub == 4096 ? part_blocks<k_part_scatter_tma<T, 4096>>(ctx->device, smem)
+                        : part_blocks<k_part_scatter_tma<T, kSub>>(ctx->device, smem);
   });
   const i64 g = std::max<i64>(1, std::min<i64>((n + rows_sub - 1) / rows_sub,
                                                (i64)ctx->num_sms * occ));
@@ -2132,7 +2156,11 @@ pq_status pq_partition(pq_ctx* ctx, pq_col key, const pq_col* payload, int npay,
   if (!key.data || !out_key) return pqh::fail(ctx, PQ_ERR_INVALID_ARG, "pq_partition: null key");
   // Many buckets: two stable passes, by the low half of the bucket number into
   // scratch and by the high half into the output, when the scratch fits.
-  if (part_two_passes(log2P, n, key, payload, npay)) {
+  // Not while the stream is being captured: scratch is then kept for the
+  // graph's replays, and a second copy of the rows is too much to keep.
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (part_two_passes(log2P, n, key, payload, npay) &&
+      cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone) {
     pqh::Scratch scr(ctx, s);
     size_t bytes = 0;
     auto put = [&](int type) {
@@ -2270,13 +2298,16 @@ pq_status pq_join_probe(pq_ctx* ctx, const pq_ht* ht, pq_col probe_key, int64_t*
   PQ_CUDA(ctx, cudaMemsetAsync(d_count, 0, sizeof(int64_t), s));
   if (probe_key.n == 0) return PQ_OK;
   PQ_DISPATCH_T(probe_key.type, TK, {
-    static const int occ = std::max(1, resident_blocks256((const void*)k_ht_probe<TK>));
-    const int grid = (int)std::min<i64>((probe_key.n + 511) / 512, (i64)ctx->num_sms * occ);
-    k_ht_probe<TK><<<grid, 256, 0, s>>>((const TK*)probe_key.data, probe_key.n,
-                                        (const longlong2*)ht->keys, ht->log2cap,
-                                        (const HtMeta*)ht->meta,
-                                        (i64*)out_probe_row,
-                                        (i64*)out_build_val, cap, (u64*)d_count);
+    static const int occ = std::max(1, resident_blocks256((const void*)k_ht_probe<TK, 4>));
+    const i64 wave = (i64)ctx->num_sms * occ;
+    const bool many = probe_key.n >= wave * 8 * 128 * 4;
+    const int grid = (int)std::min<i64>((probe_key.n + 511) / 512, wave);
+    auto probe = [&](auto k) {
+      k<<<grid, 256, 0, s>>>((const TK*)probe_key.data, probe_key.n, (const longlong2*)ht->keys,
+                             ht->log2cap, (const HtMeta*)ht->meta, (i64*)out_probe_row,
+                             (i64*)out_build_val, cap, (u64*)d_count);
+    };
+    many ? probe(k_ht_probe<TK, 4>) : probe(k_ht_probe<TK, 2>);
   });
   PQ_LAUNCHED(ctx);
   k_check_cap<<<1, 1, 0, s>>>((const i64*)d_count, cap, ctx->d_status);

@@ -226,6 +226,8 @@ def join_keys(rng, kind, n):
         return i - n // 3
     if kind == "two-scales":    # regions of dense ids
         return (i // 500 << 40) + i % 500
+    if kind == "dense-groups":  # even in the large, crowded in the small
+        return (i // 64) * 256 + i % 64
     if kind == "outliers":      # dense ids and a few keys far away
         k = i.copy()
         k[::1000] = rng.integers(-2**62, 2**62, size=len(k[::1000]))
@@ -244,7 +246,7 @@ def join_keys(rng, kind, n):
 
 
 @pytest.mark.parametrize("n", [N_HT - 1, N_HT, N_HT + 12_345])
-@pytest.mark.parametrize("kind", ["gap4", "gap1000", "dense", "two-scales", "outliers",
+@pytest.mark.parametrize("kind", ["gap4", "gap1000", "dense", "two-scales", "dense-groups", "outliers",
                                   "half-sparse", "random", "equal-low-bits", "repeated",
                                   "few-repeated-much"])
 def test_join_key_order(ctx, stream, n, kind):
