@@ -253,8 +253,11 @@ pq_status pq_ht_free(pq_ctx* ctx, pq_ht* ht, void* stream);
  * With `sel_in` (ascending row ids of a previous selection, `n_in` of them,
  * or *d_n_in of them if `d_n_in` is non-NULL) only those rows are tested, so
  * the result is the AND of both predicates.  `sel_out` holds n_in (or col.n)
- * ids.  Single pass: one read of the column, decoupled look-back for the
- * tile offsets (Merrill & Garland 2016) whose waits are bounded. */
+ * ids.  The column is read once: a first pass keeps one bit per row (n / 8
+ * bytes of scratch) and counts, a second writes the ids; up to 16384 rows
+ * take one block and no scratch.  Without room for the bits a single pass
+ * with decoupled look-back for the tile offsets (Merrill & Garland 2016),
+ * whose waits are bounded, takes its place. */
 pq_status pq_filter(pq_ctx* ctx, pq_col col, int op, int64_t c, const int64_t* sel_in,
                     int64_t n_in, const int64_t* d_n_in, int64_t* sel_out, int64_t* d_count,
                     void* stream);
@@ -263,19 +266,22 @@ pq_status pq_filter(pq_ctx* ctx, pq_col col, int op, int64_t c, const int64_t* s
  * Sec. 3.1): bucket(k) = (uint64(k) * 0x9E3779B97F4A7C15 mod 2^64)
  * >> (64 - log2P) (Fibonacci hashing; bucket 0 when log2P = 0).  Rows are
  * written to out_key / out_payload[j] grouped by bucket, in input order
- * within a bucket (stable); d_offsets[b] .. d_offsets[b+1] (device, P + 1
- * int64) delimit bucket b.  0 <= log2P <= PQ_MAX_LOG2P, npay <=
- * PQ_MAX_PAYLOAD, payload columns have key.n rows; output arrays have the
- * element types of their inputs. */
+ * within a bucket (stable; many buckets of many rows are taken in two passes
+ * outside stream capture, when the scratch holds a copy of the rows);
+ * d_offsets[b] .. d_offsets[b+1] (device, P + 1 int64) delimit bucket b.
+ * 0 <= log2P <= PQ_MAX_LOG2P, npay <= PQ_MAX_PAYLOAD, payload columns have
+ * key.n rows; output arrays have the element types of their inputs. */
 pq_status pq_partition(pq_ctx* ctx, pq_col key, const pq_col* payload, int npay, int log2P,
                        void* out_key, void* const* out_payload, int64_t* d_offsets,
                        void* stream);
 
 /* Hash-join build on the materialised left side (Sec. 3.1, 3.2): an
- * open-addressing table (linear probing, power-of-two capacity >= n /
- * load_factor) of (key, value) pairs in the arena.  `val` may have data NULL
- * (value = build row id); otherwise val.n == key.n.  Duplicate keys occupy
- * one slot each.  load_factor <= 0 takes the context default. */
+ * open-addressing table (power-of-two capacity >= n / load_factor) of (key,
+ * value) pairs in the arena, probed line by line (8 slots).  A key's first
+ * line comes from its hash or, for 2^18 build rows or more of which a sample
+ * shows keys spread evenly over their range, follows the key order.  `val`
+ * may have data NULL (value = build row id); otherwise val.n == key.n.
+ * Duplicate keys occupy one slot each.  load_factor <= 0 takes the context default. */
 pq_status pq_join_build(pq_ctx* ctx, pq_col key, pq_col val, float load_factor, pq_ht** out,
                         void* stream);
 
@@ -292,9 +298,9 @@ pq_status pq_join_probe(pq_ctx* ctx, const pq_ht* ht, pq_col probe_key, int64_t*
  * more (outside stream capture) are first looked over (key order and range),
  * which waits for the stream once: keys in ascending order, but for one late
  * part at most, are grouped by their runs with no table; otherwise, when the
- * range is at most 4 keys per row and the rows come in runs (or the slots
- * take less memory than the hash table), the groups are summed in a slot
- * array over the range. */
+ * range is at most 4 keys per row, the groups are summed in a slot array over
+ * the range -- or, for rows in no order, in the hash table when that takes
+ * less memory, and again in the slot array if it does not hold them. */
 pq_status pq_groupby_sum(pq_ctx* ctx, pq_col key, pq_col val, int64_t* out_keys,
                          int64_t* out_sums, int64_t cap, int64_t* d_ngroups, void* stream);
 

@@ -1223,6 +1223,7 @@ struct GbSummary {
   i64 runs;         // runs of equal keys
   i64 first;        // runs before the first descent (all of them: no descent)
   i64 descents;     // rows whose key is below the row's before
+  u32 over;         // the hash table did not hold the groups
 };
 struct GbWarp {
   u32 runs, before, descents;  // of the warp's rows; before its first descent
@@ -1520,28 +1521,36 @@ __device__ __forceinline__ void gb_each_run(const TK* __restrict__ key, const TV
 // rows took the dense path to 3.3 ms, the hash table to 2.7 ms).
 constexpr int kGbHotLog2 = 11;
 
-// Hash table of {key, sum} slots, one sector per run.
+// Hash table of {key, sum} slots, one sector per run.  With `over`, a table
+// that fills up is given up instead of reported: a key that finds no slot
+// within kGbMaxProbes sets the flag, and the others stop looking a line (8
+// slots) further on, so that the whole pass costs no more than a few lines a
+// row.
+constexpr u64 kGbMaxProbes = 1024;
 template <typename TK, typename TV, bool VEC>
 __global__ void __launch_bounds__(256) k_gb_insert(const TK* __restrict__ key,
                                                    const TV* __restrict__ val, i64 n,
                                                    i64* __restrict__ slots, int log2cap,
-                                                   DevStatus* st) {
+                                                   DevStatus* st, u32* over) {
   __shared__ HotSums<kGbHotLog2> hot;
   hot.clear();
   __syncthreads();
   const u64 mask = (1ULL << log2cap) - 1;
+  const u64 limit = over ? min(mask, kGbMaxProbes - 1) : mask;
   const bool use_hot = log2cap < 32;
   gb_each_run<TK, TV, VEC>(key, val, n, st, [&](i64 k, i64 acc) {
     u64 s = slot_hash(k) & mask;
     u64 probes = 0;
-    for (; probes <= mask; ++probes) {
+    for (; probes <= limit; ++probes) {
       i64 cur = slots[2 * s];  // a stale free slot is seen by the CAS
       if (cur == kEmpty) cur = (i64)atomicCAS((u64*)&slots[2 * s], (u64)kEmpty, (u64)k);
       if (cur == kEmpty || cur == k) break;
+      if (over && (probes & 7) == 7 && *(volatile u32*)over) return;
       s = (s + 1) & mask;
     }
-    if (probes > mask) {
-      latch(st, PQ_ERR_CAPACITY, -1);
+    if (probes > limit) {
+      if (over) *(volatile u32*)over = 1;
+      else latch(st, PQ_ERR_CAPACITY, -1);
       return;
     }
     if (use_hot && hot.add((u32)s, acc, hot.owner((u32)s))) return;
@@ -1559,6 +1568,15 @@ __global__ void k_gb_clear(longlong2* __restrict__ p, i64 n) {
     p[i] = make_longlong2(kEmpty, 0);
 }
 
+// The slot array's kernels take `if_over`: with it they run only if the flag
+// is set (the hash table before them did not hold the groups).
+__global__ void k_gb_zero_if(longlong2* __restrict__ p, i64 n, const u32* if_over) {
+  if (!*if_over) return;
+  const i64 stride = (i64)gridDim.x * blockDim.x;
+  for (i64 i = (i64)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride)
+    p[i] = make_longlong2(0, 0);
+}
+
 // Dense keys (a key range of at most 4 rows per key): the group of key k is
 // slot k - min, its sum in a zeroed array and its existence in a bitmap, so
 // a run costs one reduction and one bit, at addresses that follow the key
@@ -1567,7 +1585,9 @@ template <typename TK, typename TV, bool VEC>
 __global__ void __launch_bounds__(256) k_gb_dense(const TK* __restrict__ key,
                                                   const TV* __restrict__ val, i64 n, u64 umin,
                                                   u64 span, i64* __restrict__ sums,
-                                                  u32* __restrict__ bm, DevStatus* st) {
+                                                  u32* __restrict__ bm, DevStatus* st,
+                                                  const u32* if_over) {
+  if (if_over && !*if_over) return;
   __shared__ HotSums<kGbHotLog2> hot;
   hot.clear();
   __syncthreads();
@@ -1610,7 +1630,8 @@ __global__ void __launch_bounds__(256) k_gb_dense_emit(const u32* __restrict__ b
                                                        const i64* __restrict__ sums, u64 span,
                                                        u64 umin, i64* __restrict__ out_keys,
                                                        i64* __restrict__ out_sums, i64 cap,
-                                                       u64* d_ngroups) {
+                                                       u64* d_ngroups, const u32* if_over) {
+  if (if_over && !*if_over) return;
   const i64 words = (i64)((span + 31) / 32);
   const i64 stride = (i64)gridDim.x * blockDim.x;
   for (i64 w0 = (i64)blockIdx.x * blockDim.x; w0 < words; w0 += stride) {  // block-uniform
@@ -1639,7 +1660,8 @@ constexpr int kGbEmitPer = 8;
 __global__ void __launch_bounds__(256) k_gb_emit(const longlong2* __restrict__ tab, i64 slots,
                                                  i64* __restrict__ out_keys,
                                                  i64* __restrict__ out_sums, i64 cap,
-                                                 u64* d_ngroups) {
+                                                 u64* d_ngroups, const u32* over) {
+  if (over && *over) return;
   const i64 step = (i64)gridDim.x * blockDim.x * kGbEmitPer;
   for (i64 b0 = (i64)blockIdx.x * blockDim.x * kGbEmitPer; b0 < slots; b0 += step) {  // block-uniform
     const i64 b = b0 + (i64)threadIdx.x * kGbEmitPer;
@@ -2330,7 +2352,32 @@ pq_status pq_groupby_sum(pq_ctx* ctx, pq_col key, pq_col val, int64_t* out_keys,
   const i64 slots = (i64)1 << log2cap;
   pqh::Scratch tscr(ctx, s);
   auto table = [&]() { return (i64*)tscr.get((size_t)slots * 16); };
-  i64* tab = nullptr;
+  // Clear and fill the hash table.  At least 128 rows per warp; few rows are
+  // not worth a block each.
+  const int grid = (int)std::min<i64>((key.n + 1023) / 1024, (i64)ctx->num_sms * 6);
+  auto insert = [&](i64* tab, u32* over) -> pq_status {
+    k_gb_clear<<<(int)std::min<i64>((slots + 255) / 256, (i64)ctx->num_sms * 8), 256, 0, s>>>(
+        (longlong2*)tab, slots);
+    PQ_LAUNCHED(ctx);
+    PQ_DISPATCH_T(key.type, TK, {
+      PQ_DISPATCH_T(val.type, TV, {
+        auto ins = [&](auto k) {
+          k<<<grid, 256, 0, s>>>((const TK*)key.data, (const TV*)val.data, key.n, tab, log2cap,
+                                 ctx->d_status, over);
+        };
+        vec ? ins(k_gb_insert<TK, TV, true>) : ins(k_gb_insert<TK, TV, false>);
+      });
+    });
+    PQ_LAUNCHED(ctx);
+    return PQ_OK;
+  };
+  auto emit = [&](const i64* tab, const u32* over) -> pq_status {
+    const int g = (int)std::min<i64>((slots + 2047) / 2048, (i64)ctx->num_sms * 8);
+    k_gb_emit<<<g, 256, 0, s>>>((const longlong2*)tab, slots, (i64*)out_keys, (i64*)out_sums, cap,
+                                (u64*)d_ngroups, over);
+    PQ_LAUNCHED(ctx);
+    return PQ_OK;
+  };
   // Large inputs outside stream capture: one read of the keys and one small
   // read-back tell whether they come in order (groups are then their runs),
   // and their range; dense keys take the slot array.
@@ -2389,27 +2436,37 @@ pq_status pq_groupby_sum(pq_ctx* ctx, pq_col key, pq_col val, int64_t* out_keys,
           return PQ_OK;
         }
       }
-      // Rows in no order touch their groups at random: what counts is how
-      // much memory the groups take (30M Zipf rows, 7.5M groups in a range of
-      // 30M: slot array of 240 MB 0.94 ms, hash table of 134 MB 0.45 ms).
-      // Rows in runs follow the slot array's order.
       const u64 span = m.umax >= m.umin ? m.umax - m.umin + 1 : 0;
-      const bool dense_ok = span && span <= 4 * (u64)key.n && span <= (1ULL << 34);
-      if (dense_ok && (m.runs <= key.n / 2 || span <= (u64)slots || !(tab = table()))) {
+      if (span && span <= 4 * (u64)key.n && span <= (1ULL << 34)) {
         pqh::Scratch scr(ctx, s);
         const size_t sb = (size_t)((span * 8 + 255) / 256 * 256);
         const size_t bb = (size_t)(((span + 31) / 32 * 4 + 255) / 256 * 256);
         char* blk = (char*)scr.get(sb + bb);
         if (blk) {
+          // Rows in no order touch their groups at random: what counts is how
+          // much memory the groups take (30M Zipf rows, 7.5M groups in a range
+          // of 30M: slot array of 240 MB 0.94 ms, hash table of 134 MB 0.45
+          // ms).  Rows in runs follow the slot array's order.  The hash table
+          // holds `cap` groups; the slot array takes over, decided on the
+          // device, when there are more, as every group is counted.
+          i64* const tab = m.runs > key.n / 2 && span > (u64)slots ? table() : nullptr;
+          u32* const over = tab ? &sum->over : nullptr;
           i64* sums = (i64*)blk;
           u32* bm = (u32*)(blk + sb);
-          PQ_CUDA(ctx, cudaMemsetAsync(blk, 0, sb + bb, s));
-          const int gd = (int)std::min<i64>((key.n + 1023) / 1024, (i64)ctx->num_sms * 6);
+          if (tab) {
+            const pq_status st = insert(tab, over);
+            if (st != PQ_OK) return st;
+            k_gb_zero_if<<<ctx->num_sms * 8, 256, 0, s>>>((longlong2*)blk, (i64)((sb + bb) / 16),
+                                                          over);
+            PQ_LAUNCHED(ctx);
+          } else {
+            PQ_CUDA(ctx, cudaMemsetAsync(blk, 0, sb + bb, s));
+          }
           PQ_DISPATCH_T(key.type, TK, {
             PQ_DISPATCH_T(val.type, TV, {
               auto dense = [&](auto k) {
-                k<<<gd, 256, 0, s>>>((const TK*)key.data, (const TV*)val.data, key.n, m.umin, span,
-                                     sums, bm, ctx->d_status);
+                k<<<grid, 256, 0, s>>>((const TK*)key.data, (const TV*)val.data, key.n, m.umin,
+                                       span, sums, bm, ctx->d_status, over);
               };
               vec ? dense(k_gb_dense<TK, TV, true>) : dense(k_gb_dense<TK, TV, false>);
             });
@@ -2418,8 +2475,12 @@ pq_status pq_groupby_sum(pq_ctx* ctx, pq_col key, pq_col val, int64_t* out_keys,
           const i64 words = (i64)((span + 31) / 32);
           const int ge = (int)std::max<i64>(1, std::min<i64>((words + 255) / 256, (i64)ctx->num_sms * 8));
           k_gb_dense_emit<<<ge, 256, 0, s>>>(bm, sums, span, m.umin, (i64*)out_keys,
-                                             (i64*)out_sums, cap, (u64*)d_ngroups);
+                                             (i64*)out_sums, cap, (u64*)d_ngroups, over);
           PQ_LAUNCHED(ctx);
+          if (tab) {
+            const pq_status st = emit(tab, over);
+            if (st != PQ_OK) return st;
+          }
           k_check_cap<<<1, 1, 0, s>>>((const i64*)d_ngroups, cap, ctx->d_status);
           PQ_LAUNCHED(ctx);
           return PQ_OK;
@@ -2427,28 +2488,12 @@ pq_status pq_groupby_sum(pq_ctx* ctx, pq_col key, pq_col val, int64_t* out_keys,
       }
     }
   }
-  if (!tab) tab = table();
+  i64* const tab = table();
   if (!tab) return pqh::fail(ctx, PQ_ERR_BUDGET, "pq_groupby_sum: table of %lld slots",
                              (long long)slots);
-  k_gb_clear<<<(int)std::min<i64>((slots + 255) / 256, (i64)ctx->num_sms * 8), 256, 0, s>>>(
-      (longlong2*)tab, slots);
-  PQ_LAUNCHED(ctx);
-  // At least 128 rows per warp; few rows are not worth a block each.
-  const int grid = (int)std::min<i64>((key.n + 1023) / 1024, (i64)ctx->num_sms * 6);
-  PQ_DISPATCH_T(key.type, TK, {
-    PQ_DISPATCH_T(val.type, TV, {
-      auto ins = [&](auto k) {
-        k<<<grid, 256, 0, s>>>((const TK*)key.data, (const TV*)val.data, key.n, tab, log2cap,
-                               ctx->d_status);
-      };
-      vec ? ins(k_gb_insert<TK, TV, true>) : ins(k_gb_insert<TK, TV, false>);
-    });
-  });
-  PQ_LAUNCHED(ctx);
-  const int grid2 = (int)std::min<i64>((slots + 2047) / 2048, (i64)ctx->num_sms * 8);
-  k_gb_emit<<<grid2, 256, 0, s>>>((const longlong2*)tab, slots, (i64*)out_keys, (i64*)out_sums,
-                                  cap, (u64*)d_ngroups);
-  PQ_LAUNCHED(ctx);
+  pq_status st = insert(tab, nullptr);
+  if (st == PQ_OK) st = emit(tab, nullptr);
+  if (st != PQ_OK) return st;
   k_check_cap<<<1, 1, 0, s>>>((const i64*)d_ngroups, cap, ctx->d_status);
   PQ_LAUNCHED(ctx);
   return PQ_OK;

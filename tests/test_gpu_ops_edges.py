@@ -184,6 +184,34 @@ def test_groupby_capacity_is_counted(ctx, stream, order):
     assert e.value.status == pq.PQ_ERR_CAPACITY and int(ng.item()) == groups
 
 
+@pytest.mark.parametrize("cap", [1, 1000, "half", "less one", "groups", "more"])
+def test_groupby_unordered_range_above_the_table(ctx, stream, cap):
+    """Keys in no order over a range of 4 keys per row: a hash table sized for
+    cap groups, whose place the slot array takes when there are more."""
+    rng = np.random.default_rng(23)
+    n = N_GB + 77
+    k = rng.integers(0, n // 8, size=n) * 32 - 5_000_000
+    v = rng.integers(-10**9, 10**9, size=n)
+    wk, ws, _ = oracle.groupby_sum(k, v)
+    groups = len(wk)
+    cap = {"half": groups // 2, "less one": groups - 1, "groups": groups,
+           "more": groups + 100}.get(cap, cap)
+    with torch.cuda.stream(stream):
+        ok, os_, ng = pq.pq_groupby_sum(ctx, dev(k), dev(v), cap=cap, stream=stream)
+        if cap < groups:
+            with pytest.raises(pq.PQError) as e:
+                ctx.sync(stream)
+            assert e.value.status == pq.PQ_ERR_CAPACITY
+        else:
+            ctx.sync(stream)
+    assert int(ng.item()) == groups
+    m = min(cap, groups)
+    gk, gs = ok[:m].cpu().numpy(), os_[:m].cpu().numpy()
+    at = np.searchsorted(wk, gk)
+    assert len(np.unique(gk)) == m
+    assert np.array_equal(wk[at], gk) and np.array_equal(ws[at], gs)
+
+
 def test_groupby_reserved_key_in_order(ctx, stream):
     k = np.sort(np.random.default_rng(1).integers(-50, 50, size=N_GB))
     k[0] = np.iinfo(np.int64).min
