@@ -382,6 +382,14 @@ constexpr i64 kDirectShare = 8;
 // The M scan's verdict (Batch::direct_ok plans): a word of the work area, so
 // that the later kernels know it after a single load.
 constexpr int kDirectWord = 32;
+// The verdict and the phase's tile count, both asked for before either is
+// waited for (one after the other cost every kernel of a plan that does not
+// take the pass 0.7 us).
+__device__ __forceinline__ bool direct_verdict(const Batch& b, const i64* tiles, i64& total) {
+  const u32 w = b.direct_ok ? *(volatile const u32*)(b.work + kDirectWord) : 0;
+  total = *(volatile const i64*)tiles;
+  return w != 0;
+}
 // Its rank records: per 32-bit word of the M bitmap the word and the number
 // of set bits before it, so that a rank is one 8-byte load.  They take the
 // place of the hit list.
@@ -1447,10 +1455,11 @@ __global__ void __launch_bounds__(256) k_plan_mrank(Batch b) {
 __global__ void __launch_bounds__(256) k_plan_mdup(Batch b) {
   chain_begin();
   const i64* pre = b.dyn + 6 * (b.nq + 1);
-  const i64 total = pre[b.nq];
+  i64 total;
+  const bool direct = direct_verdict(b, pre + b.nq, total);
   const int lane = threadIdx.x & 31;
   const u64 keep = policy_keep();
-  if (b.direct_ok && b.work[kDirectWord]) {
+  if (direct) {
     // The direct pass's rank records, four words at a time (a tile's words
     // are a multiple of 16).
     const PlanDev& q = b.q[0];
@@ -1803,8 +1812,9 @@ __global__ void __launch_bounds__(256, 4) k_plan_fscan(Batch b) {
   const u64 keep = policy_keep(), strm = policy_stream();
   const bool ov = b.ov.table == 3;
   // A plan that takes the direct pass leaves nothing to scan here.
-  const bool skip = !BUF && b.direct_ok && b.work[kDirectWord];
-  const i64 total = skip ? 0 : ov ? b.ov.tiles : b.tF[b.nq];
+  i64 total;
+  if (!BUF && direct_verdict(b, b.tF + b.nq, total)) total = 0;
+  else if (ov || BUF) total = ov ? b.ov.tiles : b.tF[b.nq];
   int cq = -1;  // plan of the rows in the ring
   u32 hh = 0, ht = 0;
   auto flush = [&](u32 cnt) {  // cnt entries from hh to plan cq's hit list
@@ -1944,13 +1954,14 @@ __global__ void __launch_bounds__(256, 4) k_plan_fscan(Batch b) {
   if (finish(b.work, kPhFscan)) {
     const i64 warps = (i64)gridDim.x * (blockDim.x >> 5);
     __shared__ u64 s_hits;  // of all plans of the batch, which share the grid
-    if (threadIdx.x == 0) s_hits = 0;
-    __syncthreads();
-    u64 mine = 0;
-    for (int qi = threadIdx.x; qi < b.nq; qi += blockDim.x) mine += (u64)ld_count(&b.q[qi].ctr->hcount);
-    if (mine) atomicAdd((unsigned long long*)&s_hits, (unsigned long long)mine);
-    __syncthreads();
-    const i64 hits = (i64)s_hits;
+    if (b.nq > 1) {  // a single plan's are read below: a second wait here is 1 us
+      if (threadIdx.x == 0) s_hits = 0;
+      __syncthreads();
+      u64 mine = 0;
+      for (int qi = threadIdx.x; qi < b.nq; qi += blockDim.x) mine += (u64)ld_count(&b.q[qi].ctr->hcount);
+      if (mine) atomicAdd((unsigned long long*)&s_hits, (unsigned long long)mine);
+      __syncthreads();
+    }
     block_prefix(b.dyn + 7 * (b.nq + 1), b.nq, [&](int qi) -> i64 {
       const PlanDev& q = b.q[qi];
       QCtr* c = q.ctr;
@@ -1958,6 +1969,7 @@ __global__ void __launch_bounds__(256, 4) k_plan_fscan(Batch b) {
       if (q.hb_cap && h > (i64)q.hb_cap) q_latch(c, b.st, PQ_ERR_CAPACITY, h);
       // Hits per probe tile: about two tiles per warp of this grid, in
       // multiples of 32, between 64 and 4096.
+      const i64 hits = b.nq > 1 ? (i64)s_hits : h;
       i64 tl = (hits / (2 * warps) + 31) / 32 * 32;
       tl = tl < 64 ? 64 : tl > 4096 ? 4096 : tl;
       c->hp_tile = tl;
@@ -2130,7 +2142,9 @@ __global__ void __launch_bounds__(256, 4) k_plan_fprobe(Batch b) {
   __shared__ i64 s_asum[kAgg];
   __shared__ i64 s_sc[8][32];
   extern __shared__ __align__(16) unsigned char s_dyn[];  // only when direct_ok
-  if (b.direct_ok && b.work[kDirectWord]) {
+  const i64* pre = b.dyn + 7 * (b.nq + 1);
+  i64 total;
+  if (direct_verdict(b, pre + b.nq, total)) {
     auto& hot = *reinterpret_cast<HotSums<kHotLog2>*>(s_dyn);
     if (b.q[0].vec) fdirect<true>(b, hot);
     else fdirect<false>(b, hot);
@@ -2142,8 +2156,6 @@ __global__ void __launch_bounds__(256, 4) k_plan_fprobe(Batch b) {
   const u64 agg_min = (u64)gridDim.x * 2048;
   const u64 keep = policy_keep();
   const bool ov = b.ov.table == 3;
-  const i64* pre = b.dyn + 7 * (b.nq + 1);
-  const i64 total = pre[b.nq];
   WarpClaim wc;
   while (true) {
     const i64 t = wc.next(b.work, kPhFprobe);
@@ -2936,13 +2948,13 @@ __device__ __noinline__ void topk_direct(const Batch& b, TopkSmem& sm) {
 __global__ void __launch_bounds__(kTKW * 32, 4) k_plan_topk(Batch b) {
   chain_begin();
   __shared__ TopkSmem sm;
-  if (b.direct_ok && b.work[kDirectWord]) {
+  const i64* pre = b.dyn + 4 * (b.nq + 1);
+  i64 total;
+  if (direct_verdict(b, pre + b.nq, total)) {
     topk_direct(b, sm);
     finish(b.work, kPhTopk);
     return;
   }
-  const i64* pre = b.dyn + 4 * (b.nq + 1);
-  const i64 total = pre[b.nq];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   TopList L;
   L.bind(sm.scr[warp]);
