@@ -553,10 +553,10 @@ template <typename T>
 __global__ void __launch_bounds__(256, 8) k_part_hist_blk(const T* __restrict__ key, i64 n,
                                                           Digit dg, u32* __restrict__ hist,
                                                           i64 g, int hsplit,
-                                                          u32* __restrict__ tot) {
+                                                          u64* __restrict__ tot) {
   extern __shared__ u32 sh[];
   // With `tot` (the first of two passes) whole buckets are counted, into tot
-  // and, added up by digit, into hist.
+  // (over all rows: 64 bits) and, added up by digit, into hist.
   const int P = tot ? 1 << dg.log2P : dg.count();
   const Digit cd = tot ? Digit(dg.log2P, 0, dg.log2P) : dg;
   for (int b = threadIdx.x; b < P; b += blockDim.x) sh[b] = 0;
@@ -596,7 +596,7 @@ __global__ void __launch_bounds__(256, 8) k_part_hist_blk(const T* __restrict__ 
     return;
   }
   for (int b = threadIdx.x; b < P; b += blockDim.x)
-    if (sh[b]) atomicAdd(&tot[b], sh[b]);
+    if (sh[b]) atomicAdd((unsigned long long*)&tot[b], (unsigned long long)sh[b]);
   // Lane l of a warp adds up a digit's buckets l, l + 32, ...
   for (int d = warp; d < dg.count(); d += 8) {
     u32 c = 0;
@@ -604,6 +604,33 @@ __global__ void __launch_bounds__(256, 8) k_part_hist_blk(const T* __restrict__ 
     c = __reduce_add_sync(kFull, c);
     if (lane == 0 && c) atomicAdd(&hist[(i64)d * g + k], c);
   }
+}
+
+// The buckets' offsets from their counts (P <= 4096: four per thread), n last.
+// One block.
+__global__ void __launch_bounds__(1024) k_part_offsets(const u64* __restrict__ tot, int P, i64 n,
+                                                       i64* __restrict__ out) {
+  __shared__ i64 s_w[32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, b0 = threadIdx.x * 4;
+  i64 v[4], sum = 0;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) v[j] = b0 + j < P ? (i64)tot[b0 + j] : 0, sum += v[j];
+  i64 x = sum;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const i64 y = __shfl_up_sync(kFull, x, o);
+    if (lane >= o) x += y;
+  }
+  if (lane == 31) s_w[warp] = x;
+  __syncthreads();
+  i64 run = x - sum;
+  for (int w = 0; w < warp; ++w) run += s_w[w];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    if (b0 + j < P) out[b0 + j] = run;
+    run += v[j];
+  }
+  if (threadIdx.x == 0) out[P] = n;
 }
 
 // Shared memory of the staged scatter for P buckets (bytes).
@@ -2040,7 +2067,7 @@ int part_blocks(int device, size_t smem) {
 // bucket.  d_offsets: the digits' offsets (or null); tot: null, or counts of
 // whole buckets to be added to (zeroed by the caller).
 pq_status part_pass(pq_ctx* ctx, pq_col key, const pq_col* payload, int npay, Digit dg,
-                    void* out_key, void* const* out_payload, i64* d_offsets, u32* tot,
+                    void* out_key, void* const* out_payload, i64* d_offsets, u64* tot,
                     cudaStream_t s) {
   const i64 n = key.n;
   const int P = dg.count();
@@ -2194,11 +2221,10 @@ pq_status pq_partition(pq_ctx* ctx, pq_col key, const pq_col* payload, int npay,
     at[0] = put(key.type);
     for (int j = 0; j < npay; ++j) at[1 + j] = put(payload[j].type);
     char* w = (char*)scr.get(bytes);
-    const size_t tot_b = (size_t)P * 4;
-    char* t = w ? (char*)scr.get(512 + tot_b) : nullptr;
-    if (t) {
-      u32* tot = (u32*)(t + 512);
-      PQ_CUDA(ctx, cudaMemsetAsync(t, 0, 512 + tot_b, s));
+    const size_t tot_b = (size_t)P * 8;
+    u64* tot = w ? (u64*)scr.get(tot_b) : nullptr;
+    if (tot) {
+      PQ_CUDA(ctx, cudaMemsetAsync(tot, 0, tot_b, s));
       const int lo = log2P / 2;
       pq_col k1 = key, p1[PQ_MAX_PAYLOAD];
       void* o1[PQ_MAX_PAYLOAD];
@@ -2210,11 +2236,9 @@ pq_status pq_partition(pq_ctx* ctx, pq_col key, const pq_col* payload, int npay,
         st = part_pass(ctx, k1, p1, npay, Digit(log2P, lo, log2P - lo), out_key, out_payload,
                        nullptr, nullptr, s);
       if (st == PQ_OK) {
-        // The buckets' offsets from their counts (P <= 4096: one tile).
-        k_scan_u32<<<1, 256, 0, s>>>(tot, P, (i64*)d_offsets, (u64*)(t + 256), (u32*)t,
-                                     ctx->opt.spin_limit, ctx->d_status);
+        k_part_offsets<<<1, 1024, 0, s>>>(tot, P, n, (i64*)d_offsets);
         PQ_LAUNCHED(ctx);
-        return pqh::fill_i64(ctx, (i64*)d_offsets + P, 1, n, s);
+        return PQ_OK;
       }
       if (st != PQ_ERR_BUDGET) return st;
     }
