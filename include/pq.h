@@ -297,7 +297,9 @@ pq_status pq_join_probe(pq_ctx* ctx, const pq_ht* ht, pq_col probe_key, int64_t*
  * hash table is sized for min(key.n, cap) groups.  Inputs of 2^20 rows or
  * more (outside stream capture) are first looked over (key order and range),
  * which waits for the stream once: keys in ascending order, but for one late
- * part at most, are grouped by their runs with no table; otherwise, when the
+ * part at most, are grouped by their runs with no table (unless an output
+ * overlaps an input, which is allowed: the other ways write after the last
+ * read); otherwise, when the
  * range is at most 4 keys per row, the groups are summed in a slot array over
  * the range -- or, for rows in no order, in the hash table when that takes
  * less memory, and again in the slot array if it does not hold them. */

@@ -1896,6 +1896,10 @@ void launch_filter_v(pq_ctx* ctx, bool vec, int grid, cudaStream_t s, const void
 
 bool aligned16(const void* p) { return ((uintptr_t)p & 15) == 0; }
 
+bool overlaps(const void* a, size_t a_bytes, const void* b, size_t b_bytes) {
+  return (uintptr_t)a < (uintptr_t)b + b_bytes && (uintptr_t)b < (uintptr_t)a + a_bytes;
+}
+
 // Blocks of 256 threads (static shared memory only) resident per SM.
 int resident_blocks256(const void* k) {
   int occ = 0;
@@ -2434,8 +2438,16 @@ pq_status pq_groupby_sum(pq_ctx* ctx, pq_col key, pq_col val, int64_t* out_keys,
       // late part appended to an ordered table); the reserved key (ukey 0)
       // goes to the tables, which report it.
       const i64 tail = m.runs - m.first;
-      if (m.umin != 0 && (m.descents == 0 ||
-                          (m.descents == 1 && tail <= key.n / 8 && m.first <= cap))) {
+      // The runs' groups are written while other rows are read: not over the
+      // inputs.  The tables write after the last read.
+      const size_t out_b = (size_t)std::min<i64>(key.n, cap) * 8;
+      bool over_inputs = false;
+      for (const pq_col& c : {key, val})
+        for (const int64_t* o : {out_keys, out_sums})
+          over_inputs |= overlaps(o, out_b, c.data, (size_t)c.n * pqh::dtype_size(c.type));
+      if (m.umin != 0 && !over_inputs && (m.descents == 0 ||
+                                          (m.descents == 1 && tail <= key.n / 8 &&
+                                           m.first <= cap))) {
         pqh::Scratch ts(ctx, s);
         i64* tk = tail ? (i64*)ts.get((size_t)tail * 16) : nullptr;
         if (!tail || tk) {
