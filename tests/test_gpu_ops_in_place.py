@@ -60,3 +60,28 @@ def test_groupby_over_its_inputs(ctx, stream, order, where):
     gk, gs = ok[:m].cpu().numpy(), os[:m].cpu().numpy()
     at = np.argsort(gk)
     assert np.array_equal(gk[at], uk) and np.array_equal(gs[at], sums)
+
+
+# One block, the sizes around it, and several tiles per block.
+@pytest.mark.parametrize("n", [300, 16_384, 16_385, 200_003, 4_000_001, 12_000_001])
+@pytest.mark.parametrize("deferred", [False, True])
+def test_filter_refines_a_selection_in_place(ctx, stream, n, deferred):
+    rng = np.random.default_rng(n)
+    a = rng.integers(0, 100, size=n).astype(np.int32)
+    sel = np.flatnonzero(rng.random(n) < 0.9).astype(np.int64)
+    buf = torch.from_numpy(np.concatenate([sel, sel[:100]])).cuda()
+    x, m = torch.from_numpy(a).cuda(), len(sel)
+    n_in = torch.tensor([m], device="cuda")
+    cnt = torch.zeros(1, dtype=torch.int64, device="cuda")
+    torch.cuda.synchronize()
+    for _ in range(3):  # later rounds drop nothing more
+        ctx.check(pq.library().pq_filter(ctx.h, pq.col(x), pq.CMP["<"], 97, buf.data_ptr(), m,
+                                         n_in.data_ptr() if deferred else None, buf.data_ptr(),
+                                         cnt.data_ptr(), stream.cuda_stream))
+        ctx.sync(stream)
+        want = sel[a[sel] < 97]
+        assert int(cnt.item()) == len(want)
+        assert np.array_equal(buf[:len(want)].cpu().numpy(), want)
+        m = len(want)
+        n_in.fill_(m)
+        torch.cuda.synchronize()
