@@ -1985,7 +1985,10 @@ pq_status pq_filter(pq_ctx* ctx, pq_col col, int op, int64_t c, const int64_t* s
   }
   const bool vec = sel ? aligned16(sel_in) : aligned16(col.data);
   const i64 wtiles = (n_cap + kWarpTile - 1) / kWarpTile;
-  if (wtiles <= kFilterOne) {
+  // A selection refined in place: only the single pass reads a tile's ids
+  // before any id is written over them.
+  const bool in_place = sel && overlaps(sel_in, (size_t)n_cap * 8, sel_out, (size_t)n_cap * 8);
+  if (wtiles <= kFilterOne && !in_place) {
     PQ_DISPATCH_T(col.type, T, {
       auto one = [&](auto k) {
         k<<<1, kFilterOne * 32, 0, s>>>((const T*)col.data, (const i64*)sel_in, n_cap,
@@ -2002,7 +2005,7 @@ pq_status pq_filter(pq_ctx* ctx, pq_col col, int op, int64_t c, const int64_t* s
   const int g = (int)std::max<i64>(1, std::min<i64>((wtiles + 15) / 16,
                                                        (i64)ctx->num_sms * filter_blocks(sel || col.type == PQ_INT64)));
   const size_t bits_b = (size_t)wtiles * 64, cnt_b = (size_t)g * 9 * 4;
-  if (char* w = (char*)scr.get(bits_b + cnt_b)) {
+  if (char* w = in_place ? nullptr : (char*)scr.get(bits_b + cnt_b)) {
     u32* block_cnt = (u32*)(w + bits_b);
     u32* warp_cnt = block_cnt + g;
     PQ_DISPATCH_T(col.type, T, {
@@ -2022,8 +2025,8 @@ pq_status pq_filter(pq_ctx* ctx, pq_col col, int op, int64_t c, const int64_t* s
     PQ_LAUNCHED(ctx);
     return PQ_OK;
   }
-  // No room for the bits (n / 8 bytes): the single pass with look-back, whose
-  // scratch is 8 bytes per 4096 rows.
+  // In place, or no room for the bits (n / 8 bytes): the single pass with
+  // look-back, whose scratch is 8 bytes per 4096 rows.
   PQ_CUDA(ctx, cudaMemsetAsync(d_count, 0, sizeof(int64_t), s));
   const i64 ntiles = (n_cap + kFilterTile - 1) / kFilterTile;
   char* w = (char*)scr.get(ntiles * 8 + 256);
