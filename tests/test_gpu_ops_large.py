@@ -16,16 +16,16 @@ def bucket(key, log2P):
 
 @pytest.mark.parametrize("log2P", [10, 12])
 def test_partition_bucket_of_more_than_2_32_rows(log2P):
-    """One key holds 2^32 rows and a few more: every offset after its bucket
-    lies beyond 2^32."""
+    """One key holds 2^32 rows and a few more (52 GB in all): every offset
+    after its bucket lies beyond 2^32."""
     n, hot, rare = 2**32 + 4099, 5, (7, -100, 31, 90)
-    key = torch.full((n,), hot, dtype=torch.int8, device="cuda")
+    key = torch.full((n,), hot, dtype=torch.int32, device="cuda")
     at = {k: 1000 * (j + 1) for j, k in enumerate(rare)}
     for k, j in at.items():
         key[j * 10:j * 10 + j] = k
     count = {**at, hot: n - sum(at.values())}
     assert len({bucket(k, log2P) for k in count}) == len(count)
-    ctx, s = pq.Context(arena_bytes=6 << 30), torch.cuda.Stream()
+    ctx, s = pq.Context(arena_bytes=17 << 30), torch.cuda.Stream()
     torch.cuda.synchronize()
     with torch.cuda.stream(s):
         out, _, off = pq.pq_partition(ctx, key, log2P=log2P, stream=s)
