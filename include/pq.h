@@ -255,7 +255,8 @@ pq_status pq_ht_free(pq_ctx* ctx, pq_ht* ht, void* stream);
  * the result is the AND of both predicates.  `sel_out` holds n_in (or col.n)
  * ids.  The column is read once: a first pass keeps one bit per row (n / 8
  * bytes of scratch) and counts, a second writes the ids; up to 16384 rows
- * take one block and no scratch.  Without room for the bits, and where
+ * take one block and no scratch.  While the stream is being captured no bits
+ * are kept and the second pass tests the rows again.  Without room for the bits, and where
  * `sel_out` is `sel_in` itself (a selection refined in place), a single pass
  * with decoupled look-back for the tile offsets (Merrill & Garland 2016),
  * whose waits are bounded, takes its place. */

@@ -138,10 +138,12 @@ __global__ void __launch_bounds__(256) k_filter(const T* __restrict__ col,
 // those of the warps before it, and from then on a warp needs only its own
 // bits: it orders the passing rows of a tile in shared memory and writes them
 // as one contiguous run.  Pass 1 is bound by reading the column, pass 2 by
-// writing the ids.  60M int32 rows, 31.5M ids out (0.49 GB): 0.188 ms with a
-// second read of the column, a scan launch between the passes and each lane
-// writing its own ids (runs with gaps: sectors written in four parts); 0.042 +
-// 0.048 ms like this, 5.4 TB/s.
+// writing the ids.  In a stream that is being captured, whose scratch is kept
+// for the graph's replays, pass 1 keeps only the counts (36 bytes per block)
+// and pass 2 tests the rows again.  60M int32 rows, 31.5M ids out (0.49 GB):
+// 0.188 ms with a second read of the column, a scan launch between the passes
+// and each lane writing its own ids (runs with gaps: sectors written in four
+// parts); 0.042 + 0.048 ms like this, 5.4 TB/s.
 constexpr int kWarpTile = 512;
 // Resident blocks per SM: 6 leave 40 registers a thread, enough for the 16
 // values of a narrow column; wide ones and row ids take 4.
@@ -278,7 +280,7 @@ __global__ void __launch_bounds__(256, filter_blocks(SEL || sizeof(T) == 8))
   u32 cnt = 0;
   for (i64 t = filter_share(ntiles, nw, gw); t < t1; ++t) {
     const u32 bits = filter_bits<T, SEL, VEC>(col, sel_in, n, pt, t * kWarpTile);
-    bits_out[t * 32 + lane] = (unsigned short)bits;
+    if (bits_out) bits_out[t * 32 + lane] = (unsigned short)bits;
     cnt += __popc(bits);
   }
   cnt = __reduce_add_sync(kFull, cnt);
@@ -292,11 +294,13 @@ __global__ void __launch_bounds__(256, filter_blocks(SEL || sizeof(T) == 8))
   }
 }
 
-template <bool SEL>
-__global__ void __launch_bounds__(256, filter_blocks(false))
-    k_filter_emit(const i64* __restrict__ sel_in, i64 n_cap, const i64* d_n,
-                  const unsigned short* __restrict__ bits_in, const u32* __restrict__ warp_cnt,
-                  const u32* __restrict__ block_cnt, i64* __restrict__ out, i64* d_count) {
+// Pass 2 of a block; bits_of(t): the lane's bits of warp tile t, asked for one
+// tile ahead.
+template <bool SEL, typename F>
+__device__ __forceinline__ void filter_emit(const i64* __restrict__ sel_in, i64 n,
+                                            const u32* __restrict__ warp_cnt,
+                                            const u32* __restrict__ block_cnt,
+                                            i64* __restrict__ out, i64* d_count, F bits_of) {
   __shared__ unsigned short s_stage[8][kWarpTile];
   __shared__ u64 s_before;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -308,7 +312,6 @@ __global__ void __launch_bounds__(256, filter_blocks(false))
   for (int o = 16; o > 0; o >>= 1) before += __shfl_xor_sync(kFull, before, o);
   if (lane == 0 && before) atomicAdd((unsigned long long*)&s_before, (unsigned long long)before);
   __syncthreads();
-  const i64 n = d_n ? min(*d_n, n_cap) : n_cap;
   const i64 ntiles = (n + kWarpTile - 1) / kWarpTile, nw = (i64)gridDim.x * 8;
   const i64 gw = (i64)blockIdx.x * 8 + warp;
   i64 pos = (i64)s_before;
@@ -316,12 +319,35 @@ __global__ void __launch_bounds__(256, filter_blocks(false))
   for (int w = 0; w < warp; ++w) pos += __ldg(warp_cnt + (i64)blockIdx.x * 8 + w);
   const i64 t1 = filter_share(ntiles, nw, gw + 1);
   i64 t = filter_share(ntiles, nw, gw);
-  u32 next = t < t1 ? __ldg(bits_in + t * 32 + lane) : 0;
+  u32 next = t < t1 ? bits_of(t) : 0;
   for (; t < t1; ++t) {
     const u32 bits = next;
-    if (t + 1 < t1) next = __ldg(bits_in + (t + 1) * 32 + lane);
+    if (t + 1 < t1) next = bits_of(t + 1);
     pos += filter_emit_tile<SEL>(bits, t * kWarpTile, sel_in, s_stage[warp], out, pos);
   }
+}
+
+template <bool SEL>
+__global__ void __launch_bounds__(256, filter_blocks(false))
+    k_filter_emit(const i64* __restrict__ sel_in, i64 n_cap, const i64* d_n,
+                  const unsigned short* __restrict__ bits_in, const u32* __restrict__ warp_cnt,
+                  const u32* __restrict__ block_cnt, i64* __restrict__ out, i64* d_count) {
+  const i64 n = d_n ? min(*d_n, n_cap) : n_cap;
+  filter_emit<SEL>(sel_in, n, warp_cnt, block_cnt, out, d_count,
+                   [&](i64 t) -> u32 { return __ldg(bits_in + t * 32 + (threadIdx.x & 31)); });
+}
+
+// Pass 2 without kept bits: the rows are tested again.
+template <typename T, bool SEL, bool VEC>
+__global__ void __launch_bounds__(256, filter_blocks(SEL || sizeof(T) == 8))
+    k_filter_again(const T* __restrict__ col, const i64* __restrict__ sel_in, i64 n_cap,
+                   const i64* d_n, Pred p, const u32* __restrict__ warp_cnt,
+                   const u32* __restrict__ block_cnt, i64* __restrict__ out, i64* d_count) {
+  const i64 n = d_n ? min(*d_n, n_cap) : n_cap;
+  const PredT<T> pt(p);
+  filter_emit<SEL>(sel_in, n, warp_cnt, block_cnt, out, d_count, [&](i64 t) -> u32 {
+    return filter_bits<T, SEL, VEC>(col, sel_in, n, pt, t * kWarpTile);
+  });
 }
 
 // Few rows (kFilterOne warp tiles): both passes in one block and one launch,
@@ -2004,24 +2030,40 @@ pq_status pq_filter(pq_ctx* ctx, pq_col col, int op, int64_t c, const int64_t* s
   // At least two warp tiles per warp, at most one wave of blocks.
   const int g = (int)std::max<i64>(1, std::min<i64>((wtiles + 15) / 16,
                                                        (i64)ctx->num_sms * filter_blocks(sel || col.type == PQ_INT64)));
-  const size_t bits_b = (size_t)wtiles * 64, cnt_b = (size_t)g * 9 * 4;
+  // Scratch of a capture is kept for the graph's replays: only the counts.
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  cudaStreamIsCapturing(s, &cap);
+  const bool keep = cap == cudaStreamCaptureStatusNone;
+  const size_t bits_b = keep ? (size_t)wtiles * 64 : 0, cnt_b = (size_t)g * 9 * 4;
   if (char* w = in_place ? nullptr : (char*)scr.get(bits_b + cnt_b)) {
+    unsigned short* bits = keep ? (unsigned short*)w : nullptr;
     u32* block_cnt = (u32*)(w + bits_b);
     u32* warp_cnt = block_cnt + g;
     PQ_DISPATCH_T(col.type, T, {
       auto mark = [&](auto k) {
         k<<<g, 256, 0, s>>>((const T*)col.data, (const i64*)sel_in, n_cap, (const i64*)d_n_in, p,
-                            (unsigned short*)w, warp_cnt, block_cnt);
+                            bits, warp_cnt, block_cnt);
       };
       if (sel) vec ? mark(k_filter_mark<T, true, true>) : mark(k_filter_mark<T, true, false>);
       else vec ? mark(k_filter_mark<T, false, true>) : mark(k_filter_mark<T, false, false>);
     });
     PQ_LAUNCHED(ctx);
-    auto emit = [&](auto k) {
-      k<<<g, 256, 0, s>>>((const i64*)sel_in, n_cap, (const i64*)d_n_in, (const unsigned short*)w,
-                          warp_cnt, block_cnt, (i64*)sel_out, (i64*)d_count);
-    };
-    sel ? emit(k_filter_emit<true>) : emit(k_filter_emit<false>);
+    if (keep) {
+      auto emit = [&](auto k) {
+        k<<<g, 256, 0, s>>>((const i64*)sel_in, n_cap, (const i64*)d_n_in, bits, warp_cnt,
+                            block_cnt, (i64*)sel_out, (i64*)d_count);
+      };
+      sel ? emit(k_filter_emit<true>) : emit(k_filter_emit<false>);
+    } else {
+      PQ_DISPATCH_T(col.type, T, {
+        auto again = [&](auto k) {
+          k<<<g, 256, 0, s>>>((const T*)col.data, (const i64*)sel_in, n_cap, (const i64*)d_n_in,
+                              p, warp_cnt, block_cnt, (i64*)sel_out, (i64*)d_count);
+        };
+        if (sel) vec ? again(k_filter_again<T, true, true>) : again(k_filter_again<T, true, false>);
+        else vec ? again(k_filter_again<T, false, true>) : again(k_filter_again<T, false, false>);
+      });
+    }
     PQ_LAUNCHED(ctx);
     return PQ_OK;
   }
