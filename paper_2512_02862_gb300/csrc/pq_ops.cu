@@ -1029,8 +1029,8 @@ __global__ void __launch_bounds__(256, 3) k_part_scatter_tma(i64 n, Digit dg,
 // ========================================================== hash join ====
 // The join's hash table: 2^log2cap slots of 16 bytes, {key, value} side by
 // side, in lines of 8 (128 bytes).  A key's slots are its line's, in turn from
-// its first one, and when the line is full, slots from the key's hash on, one
-// after another.  Where the build keys lie evenly in their range (k_ht_spread
+// its first one, and when the line is full, those of other lines from the
+// key's hash on.  Where the build keys lie evenly in their range (k_ht_spread
 // looks at a sample), line and first slot follow the key order, as many
 // lines as the range has parts: keys built or probed in order then go
 // through a line together, where hashed ones go to a sector of their own
@@ -1043,24 +1043,25 @@ struct HtMeta {
   u64 umin, range;  // the sample's smallest key (ukey) and its last key's distance
   u64 scale;        // slots per key distance, in 2^-64 (0: hashed)
 };
-struct HtPath {
-  u64 line, pos;
-};
-__device__ __forceinline__ HtPath ht_path(const HtMeta& m, i64 k, u64 mask) {
+// A key's path: its first slot, the other slots of that line in turn, and, as
+// long as lines are full, lines from the key's hash on, an odd number of lines
+// near the golden section of the table apart (so each line is met once, and a
+// few steps leave any part of the table).  Keys that crowd one part of a table
+// in key order so spread over all of it: taken slot after slot from the hash
+// on, a path that met a full part had to walk through it (2M keys, a quarter
+// of them in a twelfth of the range: paths of up to 346211 slots, 422 on
+// average; like this the longest has 21).
+__device__ __forceinline__ u64 ht_first(const HtMeta& m, i64 k, u64 mask) {
   const u64 d = ((u64)k ^ 0x8000000000000000ULL) - m.umin;
-  HtPath p;
-  if (m.scale && d <= m.range) {  // m.scale is warp-uniform
-    const u64 q = __umul64hi(d, m.scale);
-    p.line = q & ~7ULL, p.pos = q & 7;
-  } else {
-    const u64 h = slot_hash(k);
-    p.line = h & mask & ~7ULL, p.pos = h & 7;
-  }
-  return p;
+  // m.scale is warp-uniform
+  return m.scale && d <= m.range ? __umul64hi(d, m.scale) : slot_hash(k) & mask;
 }
-// The i-th slot of key k's path.
-__device__ __forceinline__ u64 ht_slot(const HtPath& p, i64 k, u64 i, u64 mask) {
-  return i < 8 ? p.line + ((p.pos + i) & 7) : ((slot_hash(k) >> 20) + i - 8) & mask;
+// Slot i of the path from slot i - 1.
+__device__ __forceinline__ u64 ht_next(u64 s, i64 k, u64 i, u64 mask) {
+  const u64 pos = (s + 1) & 7;
+  if (i & 7) return (s & ~7ULL) | pos;
+  const u64 step = __umul64hi(0x9E3779B97F4A7C15ULL, (mask + 1) >> 3) | 1;
+  return (((slot_hash(k) >> 20) + (i - 8) * step) & mask & ~7ULL) | pos;
 }
 
 // 512 build keys spread over the input (the first and the last among them):
@@ -1125,7 +1126,6 @@ __global__ void __launch_bounds__(256) k_ht_build(const TK* __restrict__ key, co
   for (i64 i0 = (i64)blockIdx.x * blockDim.x + threadIdx.x; i0 < n; i0 += kBldKeys * stride) {
     i64 k[kBldKeys], v[kBldKeys], old[kBldKeys];
     u64 s[kBldKeys];
-    HtPath p[kBldKeys];
 #pragma unroll
     for (int h = 0; h < kBldKeys; ++h) {
       const i64 i = i0 + h * stride;
@@ -1135,8 +1135,7 @@ __global__ void __launch_bounds__(256) k_ht_build(const TK* __restrict__ key, co
     }
 #pragma unroll
     for (int h = 0; h < kBldKeys; ++h) {
-      p[h] = ht_path(m, k[h], mask);
-      s[h] = ht_slot(p[h], k[h], 0, mask);
+      s[h] = ht_first(m, k[h], mask);
       old[h] = kEmpty;
       if (k[h] != kEmpty) old[h] = (i64)atomicCAS((u64*)&slots[2 * s[h]], (u64)kEmpty, (u64)k[h]);
     }
@@ -1147,7 +1146,7 @@ __global__ void __launch_bounds__(256) k_ht_build(const TK* __restrict__ key, co
       while (old[h] != kEmpty) {
         if (old[h] == k[h]) meta->dup = 1;
         if (++probes > mask + 8) break;
-        s[h] = ht_slot(p[h], k[h], probes, mask);
+        s[h] = ht_next(s[h], k[h], probes, mask);
         old[h] = (i64)atomicCAS((u64*)&slots[2 * s[h]], (u64)kEmpty, (u64)k[h]);
       }
       if (old[h] == kEmpty) slots[2 * s[h] + 1] = v[h];
@@ -1201,14 +1200,14 @@ __global__ void __launch_bounds__(256, 4) k_ht_probe(const TK* __restrict__ pkey
   for (i64 wb = gw * (32 * ROWS); wb < n; wb += nwarps * (32 * ROWS)) {
     i64 i[ROWS], k[ROWS];
     bool active[ROWS];
-    HtPath p[ROWS];
+    u64 s[ROWS];
 #pragma unroll
     for (int h = 0; h < ROWS; ++h) {
       i[h] = wb + h * 32 + lane;
       active[h] = i[h] < n;
       k[h] = active[h] ? (i64)__ldg(pkey + i[h]) : 0;
       if (k[h] == kEmpty) active[h] = false;
-      p[h] = ht_path(m, k[h], mask);
+      s[h] = ht_first(m, k[h], mask);
     }
     for (u64 j = 0; j <= mask + 8; ++j) {  // (a table with no free slot: the path ends)
       bool any = false;
@@ -1218,18 +1217,18 @@ __global__ void __launch_bounds__(256, 4) k_ht_probe(const TK* __restrict__ pkey
       longlong2 kv[ROWS];  // {key, value} of each row's current slot
 #pragma unroll
       for (int h = 0; h < ROWS; ++h)
-        kv[h] = active[h] ? __ldg(slots + ht_slot(p[h], k[h], j, mask)) : make_longlong2(kEmpty, 0);
+        kv[h] = active[h] ? __ldg(slots + s[h]) : make_longlong2(kEmpty, 0);
 #pragma unroll
       for (int h = 0; h < ROWS; ++h) {
         bool emit = false;
         if (active[h]) {
           if (kv[h].x == kEmpty) {
             active[h] = false;
-          } else if (kv[h].x == k[h] &&
-                     (j < 8 || (ht_slot(p[h], k[h], j, mask) & ~7ULL) != p[h].line)) {
-            emit = true;  // (the chain may come by the key's line again)
+          } else if (kv[h].x == k[h] && (j < 8 || ((s[h] ^ ht_first(m, k[h], mask)) & ~7ULL))) {
+            emit = true;  // (the path may come by the key's first line again)
             if (!dup) active[h] = false;
           }
+          s[h] = ht_next(s[h], k[h], j + 1, mask);
         }
         const u32 em = __ballot_sync(kFull, emit);
         if (emit) {
