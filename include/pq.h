@@ -278,10 +278,10 @@ pq_status pq_partition(pq_ctx* ctx, pq_col key, const pq_col* payload, int npay,
                        void* stream);
 
 /* Hash-join build on the materialised left side (Sec. 3.1, 3.2): an
- * open-addressing table (power-of-two capacity >= n / load_factor) of (key,
- * value) pairs in the arena, probed line by line (8 slots).  A key's first
- * line comes from its hash or, for 2^18 build rows or more of which a sample
- * shows keys spread evenly over their range, follows the key order.  `val`
+ * open-addressing table (linear probing, power-of-two capacity >= n /
+ * load_factor) of (key, value) pairs in the arena.  For 3 * 2^18 build rows or
+ * more of which a sample shows keys spread evenly over their range, the slots
+ * follow the key order instead of the hash, line by line (8 slots).  `val`
  * may have data NULL (value = build row id); otherwise val.n == key.n.
  * Duplicate keys occupy one slot each.  load_factor <= 0 takes the context default. */
 pq_status pq_join_build(pq_ctx* ctx, pq_col key, pq_col val, float load_factor, pq_ht** out,

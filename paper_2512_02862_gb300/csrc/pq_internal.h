@@ -327,7 +327,6 @@ struct Scratch {
 };
 
 // Launchers implemented in pq_ops.cu, used by the plan paths.
-pq_status fill_i64(pq_ctx* ctx, pqk::i64* p, int64_t n, pqk::i64 v, cudaStream_t s);
 // The top-k operator's kernel on caller-provided scratch: `ticket` zeroed
 // before the launch, `lists` topk_scratch_bytes(ctx, n, k) bytes; it always
 // writes *d_nout (n >= 1).  `chained`: programmatic dependent launch.

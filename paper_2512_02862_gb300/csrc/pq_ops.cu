@@ -368,11 +368,6 @@ __global__ void __launch_bounds__(kFilterOne * 32)
   if (cnt) filter_emit_tile<SEL>(bits, base, sel_in, s_stage[warp], out, (i64)pos);
 }
 
-__global__ void k_fill(i64* __restrict__ p, i64 n, i64 v) {
-  const i64 stride = (i64)gridDim.x * blockDim.x;
-  for (i64 i = (i64)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) p[i] = v;
-}
-
 // =========================================================== partition ====
 // 8192 rows per tile; warp w owns rows w*1024 .. w*1024+1023 of the tile and
 // walks them in 32 steps of 32 rows, so ranks assigned in step order keep the
@@ -1028,33 +1023,32 @@ __global__ void __launch_bounds__(256, 3) k_part_scatter_tma(i64 n, Digit dg,
 
 // ========================================================== hash join ====
 // The join's hash table: 2^log2cap slots of 16 bytes, {key, value} side by
-// side, in lines of 8 (128 bytes).  A key's slots are its line's, in turn from
-// its first one, and when the line is full, those of other lines from the
-// key's hash on.  Where the build keys lie evenly in their range (k_ht_spread
-// looks at a sample), line and first slot follow the key order, as many
-// lines as the range has parts: keys built or probed in order then go
-// through a line together, where hashed ones go to a sector of their own
-// each.  (Keys that start in the first half of their line only would make a
-// line cost 64 bytes, but meet each other more often: 1.39 ms for a join that
-// takes 1.30 ms.)  Otherwise line and first slot are the key's hash.
+// side, so that an insert and a match each touch one sector.  Linear probing
+// from the key's hash; or, where the build keys lie evenly in their range
+// (ht_spread looks at a sample), a first slot that follows the key order, as
+// many slots as the range has parts, and then the rest of its line of 8 (128
+// bytes): keys built or probed in order then go through a line together,
+// where hashed ones go to a sector of their own each.  Keys that are hashed
+// gain nothing from lines: 3 % of lines are full, and a warp whose 64 probes
+// wait for the longest path met one nearly every time (4M keys in no order:
+// build 154 -> 192 us, 16M probes 198 -> 261 us).
 struct HtMeta {
   i64 dup;        // a build key repeats
   i64 pad;
   u64 umin, range;  // the sample's smallest key (ukey) and its last key's distance
   u64 scale;        // slots per key distance, in 2^-64 (0: hashed)
 };
-// A key's path: its first slot, the other slots of that line in turn, and, as
-// long as lines are full, lines from the key's hash on, an odd number of lines
-// near the golden section of the table apart (so each line is met once, and a
-// few steps leave any part of the table).  Keys that crowd one part of a table
-// in key order so spread over all of it: taken slot after slot from the hash
-// on, a path that met a full part had to walk through it (2M keys, a quarter
-// of them in a twelfth of the range: paths of up to 346211 slots, 422 on
-// average; like this the longest has 21).
+// A path in key order: the first slot, the other slots of that line in turn,
+// and, as long as lines are full, lines from the key's hash on, an odd number
+// of lines near the golden section of the table apart (so each line is met
+// once, and a few steps leave any part of the table).  Keys that crowd one
+// part so spread over all of it: taken slot after slot from the hash on, a path
+// that met a full part had to walk through it (2M keys, a quarter of them in a
+// twelfth of the range: paths of up to 346211 slots, 422 on average; like this
+// the longest has 21).
 __device__ __forceinline__ u64 ht_first(const HtMeta& m, i64 k, u64 mask) {
   const u64 d = ((u64)k ^ 0x8000000000000000ULL) - m.umin;
-  // m.scale is warp-uniform
-  return m.scale && d <= m.range ? __umul64hi(d, m.scale) : slot_hash(k) & mask;
+  return d <= m.range ? __umul64hi(d, m.scale) : slot_hash(k) & mask;
 }
 // Slot i of the path from slot i - 1.
 __device__ __forceinline__ u64 ht_next(u64 s, i64 k, u64 i, u64 mask) {
@@ -1071,10 +1065,13 @@ __device__ __forceinline__ u64 ht_next(u64 s, i64 k, u64 i, u64 mask) {
 // no line gets more of them than it has slots (keys that come in dense groups
 // with gaps between them are hashed).  One block.
 constexpr int kHtSample = 512;
-constexpr i64 kHtSpreadMin = 1 << 18;  // fewer keys: the table lies in L2 whatever the order
+// Fewer keys: the table lies in L2 whatever the order.  At 1M keys in order
+// build and 4M probes take 103 us hashed and 87 us in key order, at 2^18 42 us
+// either way.
+constexpr i64 kHtSpreadMin = 3 << 18;
 template <typename TK>
-__global__ void __launch_bounds__(kHtSample) k_ht_spread(const TK* __restrict__ key, i64 n,
-                                                         int log2cap, HtMeta* meta) {
+__device__ __forceinline__ void ht_spread(const TK* __restrict__ key, i64 n, int log2cap,
+                                          HtMeta* meta) {
   __shared__ u64 s_lo, s_hi;
   __shared__ u32 s_cnt[kHtSample];
   const i64 k = (i64)__ldg(key + (i64)((double)(n - 1) / (kHtSample - 1) * threadIdx.x));
@@ -1096,7 +1093,7 @@ __global__ void __launch_bounds__(kHtSample) k_ht_spread(const TK* __restrict__ 
   int crowded = __syncthreads_or(fits && s_cnt[threadIdx.x] > 3);
   const u64 scale = per_key(8 * lines);
   for (int h = 1; h <= 2; ++h) {
-    const i64 r0 = n / 3 * h;  // r0 + 511 < n: 2^18 rows at least
+    const i64 r0 = n / 3 * h;  // r0 + 511 < n: kHtSpreadMin rows at least
     auto line = [&](i64 r) {
       const u64 d = ((u64)(i64)__ldg(key + r) ^ 0x8000000000000000ULL) - lo;
       return __umul64hi(min(d, range), scale) >> 3;
@@ -1113,15 +1110,66 @@ __global__ void __launch_bounds__(kHtSample) k_ht_spread(const TK* __restrict__ 
     meta->umin = lo, meta->range = range, meta->scale = scale;
 }
 
-// 15M keys 4i + U{0..3} in order: 0.94 ms when each was hashed by itself (a
-// random sector each), 0.255 ms like this (0.5 GB of lines read and written
-// back); one key at a time 0.6 ms.
-constexpr int kBldKeys = 2;  // keys per thread whose claims are in flight together
+// Clears the table; with `look` block 0 looks at the keys meanwhile (7 us of
+// waiting for a few loads, beside 10 us and more of writes).
+template <typename TK>
+__global__ void __launch_bounds__(kHtSample) k_ht_clear(longlong2* __restrict__ slots, int log2cap,
+                                                        const TK* __restrict__ key, i64 n,
+                                                        HtMeta* meta, int look) {
+  if (look && blockIdx.x == 0) {
+    ht_spread(key, n, log2cap, meta);
+    return;
+  }
+  const i64 stride = (i64)(gridDim.x - look) * blockDim.x;
+  for (i64 i = (i64)(blockIdx.x - look) * blockDim.x + threadIdx.x; i < 1LL << log2cap; i += stride)
+    slots[i] = make_longlong2(kEmpty, 0);
+}
+
+// Hashed: one key per thread, as many threads as fit (two claims in flight per
+// thread and half the warps: 4M keys 154 -> 240 us).  With `only` the kernel
+// leaves a table in key order to k_ht_build_spread.
 template <typename TK, typename TV>
-__global__ void __launch_bounds__(256) k_ht_build(const TK* __restrict__ key, const TV* __restrict__ val, i64 n,
-                           i64* __restrict__ slots, int log2cap, HtMeta* meta, DevStatus* st) {
+__global__ void __launch_bounds__(256) k_ht_build(const TK* __restrict__ key,
+                                                  const TV* __restrict__ val, i64 n,
+                                                  i64* __restrict__ slots, int log2cap,
+                                                  HtMeta* meta, int only, DevStatus* st) {
+  if (only && meta->scale) return;
   const u64 mask = (1ULL << log2cap) - 1;
+  const i64 stride = (i64)gridDim.x * blockDim.x;
+  for (i64 i = (i64)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
+    const i64 k = (i64)__ldg(key + i);
+    if (k == kEmpty) {
+      latch(st, PQ_ERR_RESERVED_KEY, i);
+      continue;
+    }
+    const i64 v = val ? (i64)__ldg(val + i) : i;
+    u64 s = slot_hash(k) & mask;
+    u64 probes = 0;
+    for (; probes <= mask; ++probes) {
+      const i64 old = (i64)atomicCAS((u64*)&slots[2 * s], (u64)kEmpty, (u64)k);
+      if (old == kEmpty) {
+        slots[2 * s + 1] = v;
+        break;
+      }
+      if (old == k) meta->dup = 1;
+      s = (s + 1) & mask;
+    }
+    if (probes > mask) latch(st, PQ_ERR_CAPACITY, i);
+  }
+}
+
+// In key order: two keys per thread whose claims are in flight together.  15M
+// keys 4i + U{0..3} in order: 0.97 ms hashed, 0.35 ms with its clear like this
+// (0.5 GB of lines read and written back); one key at a time 0.77 ms.
+constexpr int kBldKeys = 2;
+template <typename TK, typename TV>
+__global__ void __launch_bounds__(256) k_ht_build_spread(const TK* __restrict__ key,
+                                                         const TV* __restrict__ val, i64 n,
+                                                         i64* __restrict__ slots, int log2cap,
+                                                         HtMeta* meta, DevStatus* st) {
   const HtMeta m = *meta;
+  if (!m.scale) return;
+  const u64 mask = (1ULL << log2cap) - 1;
   const i64 stride = (i64)gridDim.x * blockDim.x;
   for (i64 i0 = (i64)blockIdx.x * blockDim.x + threadIdx.x; i0 < n; i0 += kBldKeys * stride) {
     i64 k[kBldKeys], v[kBldKeys], old[kBldKeys];
@@ -1155,33 +1203,34 @@ __global__ void __launch_bounds__(256) k_ht_build(const TK* __restrict__ key, co
   }
 }
 
-// Hash-join probe: a warp probes 128 rows at a time, four per lane, whose
+// Hash-join probe: a warp probes 64 rows at a time, two per lane, whose
 // chains of loads (key, then slot after slot of its path, every
 // matching build row when the build keys repeat) run side by side.  The
 // warp stages its matches in shared memory and writes them out kPrbBuf at a
 // time, reserving each run with one atomic on the output counter: one
 // reservation per pair-producing round would make that counter the bound
 // (millions of atomics on one address).  Blocks of 8 warps, one resident
-// wave.  60M rows in key order against 15M build keys: 0.89 ms with each key
-// hashed by itself, 0.50 ms with lines in key order (2 rows per lane: 0.55 ms).
-constexpr int kPrbBuf = 256;
-// ROWS: rows per lane in a round, 4 where every resident warp has several
-// rounds to do; 2 for fewer rows, which more warps then share (a join of 0.9M
-// probes with 225k keys: 182 us a call with 4, 164 with 2).
-template <typename TK, int ROWS>
-__global__ void __launch_bounds__(256, 4) k_ht_probe(const TK* __restrict__ pkey, i64 n,
-                                                  const longlong2* __restrict__ slots, int log2cap,
-                                                  const HtMeta* meta,
-                                                  i64* __restrict__ out_row,
-                                                  i64* __restrict__ out_val, i64 cap,
-                                                  u64* d_count) {
-  __shared__ i64 s_row[8][kPrbBuf], s_val[8][kPrbBuf];
+// wave, five of them per SM (48 registers).  60M rows in key order against
+// 15M build keys: 1.01 ms hashed, 0.55 ms with lines in key order (four rows
+// per lane at 64 registers, which the hashed loop cannot spare: 0.51 ms).  The hashed loop is a function of its own:
+// inlined with the other one it was 9 % slower, and as two kernels of which one
+// returns at once a probe took 6 us more.
+constexpr int kPrbBuf = 256, kPrbBlocks = 5;
+struct PrbStage {
+  i64 row[8][kPrbBuf], val[8][kPrbBuf];
+};
+template <typename TK, bool SPREAD>
+__device__ __forceinline__ void ht_probe(const TK* __restrict__ pkey, i64 n,
+                                         const longlong2* __restrict__ slots, int log2cap,
+                                         const HtMeta* meta, i64* __restrict__ out_row,
+                                         i64* __restrict__ out_val, i64 cap, u64* d_count,
+                                         PrbStage& stage) {
   const u64 mask = (1ULL << log2cap) - 1;
   const HtMeta m = *meta;
   const bool dup = m.dup != 0;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  i64* br = s_row[warp];
-  i64* bv = s_val[warp];
+  i64* br = stage.row[warp];
+  i64* bv = stage.val[warp];
   u32 nb = 0;  // staged pairs (warp-uniform)
   auto flush = [&]() {
     __syncwarp();
@@ -1197,38 +1246,37 @@ __global__ void __launch_bounds__(256, 4) k_ht_probe(const TK* __restrict__ pkey
   };
   const i64 gw = ((i64)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const i64 nwarps = ((i64)gridDim.x * blockDim.x) >> 5;
-  for (i64 wb = gw * (32 * ROWS); wb < n; wb += nwarps * (32 * ROWS)) {
-    i64 i[ROWS], k[ROWS];
-    bool active[ROWS];
-    u64 s[ROWS];
+  for (i64 wb = gw * 64; wb < n; wb += nwarps * 64) {
+    i64 i[2], k[2];
+    bool active[2];
+    u64 s[2];
 #pragma unroll
-    for (int h = 0; h < ROWS; ++h) {
+    for (int h = 0; h < 2; ++h) {
       i[h] = wb + h * 32 + lane;
       active[h] = i[h] < n;
       k[h] = active[h] ? (i64)__ldg(pkey + i[h]) : 0;
       if (k[h] == kEmpty) active[h] = false;
-      s[h] = ht_first(m, k[h], mask);
+      s[h] = SPREAD ? ht_first(m, k[h], mask) : slot_hash(k[h]) & mask;
     }
-    for (u64 j = 0; j <= mask + 8; ++j) {  // (a table with no free slot: the path ends)
-      bool any = false;
+    // Slot j of both rows; fresh(h, j): the slot is met for the first time,
+    // next(h, j): the one after it.
+    auto step = [&](u64 j, auto fresh, auto next) {
+      longlong2 kv[2];  // {key, value} of each row's current slot
 #pragma unroll
-      for (int h = 0; h < ROWS; ++h) any |= active[h];
-      if (!__any_sync(kFull, any)) break;
-      longlong2 kv[ROWS];  // {key, value} of each row's current slot
+      for (int h = 0; h < 2; ++h) kv[h] = active[h] ? __ldg(slots + s[h]) : make_longlong2(kEmpty, 0);
 #pragma unroll
-      for (int h = 0; h < ROWS; ++h)
-        kv[h] = active[h] ? __ldg(slots + s[h]) : make_longlong2(kEmpty, 0);
-#pragma unroll
-      for (int h = 0; h < ROWS; ++h) {
+      for (int h = 0; h < 2; ++h) {
         bool emit = false;
         if (active[h]) {
           if (kv[h].x == kEmpty) {
             active[h] = false;
-          } else if (kv[h].x == k[h] && (j < 8 || ((s[h] ^ ht_first(m, k[h], mask)) & ~7ULL))) {
-            emit = true;  // (the path may come by the key's first line again)
-            if (!dup) active[h] = false;
+          } else {
+            if (kv[h].x == k[h] && fresh(h, j)) {
+              emit = true;
+              if (!dup) active[h] = false;
+            }
+            s[h] = next(h, j);
           }
-          s[h] = ht_next(s[h], k[h], j + 1, mask);
         }
         const u32 em = __ballot_sync(kFull, emit);
         if (emit) {
@@ -1237,10 +1285,40 @@ __global__ void __launch_bounds__(256, 4) k_ht_probe(const TK* __restrict__ pkey
         }
         nb += __popc(em);
       }
-      if (nb > kPrbBuf - 32 * ROWS) flush();  // room for a full round stays
+      if (nb > kPrbBuf - 64) flush();  // room for a full round stays
+    };
+    if constexpr (SPREAD) {
+      for (u64 j = 0; j <= mask + 8 && __any_sync(kFull, active[0] || active[1]); ++j)
+        step(j,
+             [&](int h, u64 jj) {  // (the path may come by the first line again)
+               return jj < 8 || ((s[h] ^ ht_first(m, k[h], mask)) & ~7ULL);
+             },
+             [&](int h, u64 jj) { return ht_next(s[h], k[h], jj + 1, mask); });
+    } else {
+      while (__any_sync(kFull, active[0] || active[1]))  // a slot is always free
+        step(0, [](int, u64) { return true; }, [&](int h, u64) { return (s[h] + 1) & mask; });
     }
   }
   if (nb) flush();
+}
+template <typename TK>
+__device__ __noinline__ void ht_probe_hashed(const TK* __restrict__ pkey, i64 n,
+                                             const longlong2* __restrict__ slots, int log2cap,
+                                             const HtMeta* meta, i64* __restrict__ out_row,
+                                             i64* __restrict__ out_val, i64 cap, u64* d_count,
+                                             PrbStage& stage) {
+  ht_probe<TK, false>(pkey, n, slots, log2cap, meta, out_row, out_val, cap, d_count, stage);
+}
+template <typename TK>
+__global__ void __launch_bounds__(256, kPrbBlocks)
+    k_ht_probe(const TK* __restrict__ pkey, i64 n, const longlong2* __restrict__ slots, int log2cap,
+               const HtMeta* meta, i64* __restrict__ out_row, i64* __restrict__ out_val, i64 cap,
+               u64* d_count) {
+  __shared__ PrbStage stage;
+  if (meta->scale)
+    ht_probe<TK, true>(pkey, n, slots, log2cap, meta, out_row, out_val, cap, d_count, stage);
+  else
+    ht_probe_hashed<TK>(pkey, n, slots, log2cap, meta, out_row, out_val, cap, d_count, stage);
 }
 
 __global__ void k_check_cap(const i64* d_count, i64 cap, DevStatus* st) {
@@ -1925,16 +2003,6 @@ bool overlaps(const void* a, size_t a_bytes, const void* b, size_t b_bytes) {
   return (uintptr_t)a < (uintptr_t)b + b_bytes && (uintptr_t)b < (uintptr_t)a + a_bytes;
 }
 
-// Blocks of 256 threads (static shared memory only) resident per SM.
-int resident_blocks256(const void* k) {
-  int occ = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, 256, 0) != cudaSuccess) {
-    cudaGetLastError();
-    occ = 1;
-  }
-  return occ;
-}
-
 }  // namespace
 
 namespace pqh {
@@ -1972,13 +2040,6 @@ cudaError_t topk_launch(pq_ctx* ctx, const int64_t* keys, const int64_t* sums, i
                             (i64*)out_sums, (i64*)d_nout, (const u64*)rec_ctr, rec);
 }
 
-pq_status fill_i64(pq_ctx* ctx, i64* p, int64_t n, i64 v, cudaStream_t s) {
-  if (n <= 0) return PQ_OK;
-  int grid = (int)std::min<i64>((n + 255) / 256, (i64)ctx->num_sms * 8);
-  k_fill<<<grid, 256, 0, s>>>(p, n, v);
-  PQ_LAUNCHED(ctx);
-  return PQ_OK;
-}
 }  // namespace pqh
 
 #define PQ_DISPATCH_T(type, T, ...)              \
@@ -2344,35 +2405,35 @@ pq_status pq_join_build(pq_ctx* ctx, pq_col key, pq_col val, float load_factor, 
   ht->vals = ht->keys + 1;
   ht->log2cap = log2cap;
   ht->n = key.n;
-  pq_status st = pqh::fill_i64(ctx, ht->keys, 2 * cap, kEmpty, s);
-  if (st == PQ_OK && cudaMemsetAsync(ht->meta, 0, 256, s) != cudaSuccess)
-    st = pqh::fail(ctx, PQ_ERR_CUDA, "memset");
   HtMeta* const meta = (HtMeta*)ht->meta;
-  if (st == PQ_OK && key.n >= kHtSpreadMin) {
-    PQ_DISPATCH_T(key.type, TK, {
-      k_ht_spread<TK><<<1, kHtSample, 0, s>>>((const TK*)key.data, key.n, log2cap, meta);
-    });
-    ctx->launches++;
-    if (cudaGetLastError() != cudaSuccess) st = pqh::fail(ctx, PQ_ERR_CUDA, "k_ht_spread launch");
-  }
-  if (st == PQ_OK && key.n > 0) {
+  // Both builds are launched where the sample decides (on the device): the one
+  // that is not meant returns at once.
+  const int look = key.n >= kHtSpreadMin;
+  const pq_status st = [&]() -> pq_status {
+    PQ_CUDA(ctx, cudaMemsetAsync(ht->meta, 0, 256, s));
+    const int gc = (int)std::min<i64>((cap + 2047) / 2048, (i64)ctx->num_sms * 4) + look;
     const int grid = (int)std::min<i64>((key.n + 255) / 256, (i64)ctx->num_sms * 8);
     PQ_DISPATCH_T(key.type, TK, {
-      if (!val.data) {
-        k_ht_build<TK, long long><<<grid, 256, 0, s>>>((const TK*)key.data, nullptr, key.n,
-                                                       ht->keys, log2cap, meta,
-                                                       ctx->d_status);
-      } else {
-        PQ_DISPATCH_T(val.type, TV, {
-          k_ht_build<TK, TV><<<grid, 256, 0, s>>>((const TK*)key.data, (const TV*)val.data,
-                                                  key.n, ht->keys, log2cap, meta,
-                                                  ctx->d_status);
-        });
-      }
+      const TK* k = (const TK*)key.data;
+      k_ht_clear<TK><<<gc, kHtSample, 0, s>>>((longlong2*)ht->keys, log2cap, k, key.n, meta, look);
+      PQ_LAUNCHED(ctx);
+      if (key.n == 0) return PQ_OK;
+      auto build = [&](auto tag) -> pq_status {
+        using TV = decltype(tag);
+        k_ht_build<TK, TV><<<grid, 256, 0, s>>>(k, (const TV*)val.data, key.n, ht->keys, log2cap,
+                                                meta, look, ctx->d_status);
+        PQ_LAUNCHED(ctx);
+        if (!look) return PQ_OK;
+        k_ht_build_spread<TK, TV><<<grid, 256, 0, s>>>(k, (const TV*)val.data, key.n, ht->keys,
+                                                       log2cap, meta, ctx->d_status);
+        PQ_LAUNCHED(ctx);
+        return PQ_OK;
+      };
+      if (!val.data) return build((long long)0);
+      PQ_DISPATCH_T(val.type, TV, { return build(TV()); });
     });
-    ctx->launches++;
-    if (cudaGetLastError() != cudaSuccess) st = pqh::fail(ctx, PQ_ERR_CUDA, "k_ht_build launch");
-  }
+    return PQ_OK;
+  }();
   if (st != PQ_OK) {
     ctx->arena.release(ht->block, s);
     delete ht;
@@ -2392,16 +2453,11 @@ pq_status pq_join_probe(pq_ctx* ctx, const pq_ht* ht, pq_col probe_key, int64_t*
   PQ_CUDA(ctx, cudaMemsetAsync(d_count, 0, sizeof(int64_t), s));
   if (probe_key.n == 0) return PQ_OK;
   PQ_DISPATCH_T(probe_key.type, TK, {
-    static const int occ = std::max(1, resident_blocks256((const void*)k_ht_probe<TK, 4>));
-    const i64 wave = (i64)ctx->num_sms * occ;
-    const bool many = probe_key.n >= wave * 8 * 128 * 4;
-    const int grid = (int)std::min<i64>((probe_key.n + 511) / 512, wave);
-    auto probe = [&](auto k) {
-      k<<<grid, 256, 0, s>>>((const TK*)probe_key.data, probe_key.n, (const longlong2*)ht->keys,
-                             ht->log2cap, (const HtMeta*)ht->meta, (i64*)out_probe_row,
-                             (i64*)out_build_val, cap, (u64*)d_count);
-    };
-    many ? probe(k_ht_probe<TK, 4>) : probe(k_ht_probe<TK, 2>);
+    const int grid = (int)std::min<i64>((probe_key.n + 511) / 512, (i64)ctx->num_sms * kPrbBlocks);
+    k_ht_probe<TK><<<grid, 256, 0, s>>>((const TK*)probe_key.data, probe_key.n,
+                                        (const longlong2*)ht->keys, ht->log2cap,
+                                        (const HtMeta*)ht->meta, (i64*)out_probe_row,
+                                        (i64*)out_build_val, cap, (u64*)d_count);
   });
   PQ_LAUNCHED(ctx);
   k_check_cap<<<1, 1, 0, s>>>((const i64*)d_count, cap, ctx->d_status);

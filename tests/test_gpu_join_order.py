@@ -72,3 +72,51 @@ def test_keys_crowded_in_one_part(ctx, stream, load_factor):
     probe = np.concatenate([build[rng.integers(0, n, size=1_000_000)],
                             rng.integers(-100, n * 40 + 100, size=1_000_000)])
     check_join(ctx, stream, build, vals, probe, load_factor=load_factor)
+
+
+# Below and from the size on where a sample is taken; in key order, in no
+# order, dense; with repeated keys; 4 or 8 bytes; a few million probes, some
+# without a match.
+@pytest.mark.parametrize("n", [3 * 2**18 - 1, 3 * 2**18, 1_200_007])
+@pytest.mark.parametrize("kind", ["even", "even-int32", "dense", "shuffled", "repeated",
+                                  "repeated-shuffled"])
+def test_layouts(ctx, stream, n, kind):
+    rng = np.random.default_rng(n)
+    build = np.arange(n) * (1 if kind == "dense" else 5) - 1_000_000
+    if kind != "dense":
+        build += rng.integers(0, 5, size=n)
+    if kind.startswith("repeated"):
+        build[1::7] = build[::7][:len(build[1::7])]
+    if kind.endswith("shuffled"):
+        rng.shuffle(build)
+    probe = rng.integers(build.min() - 1000, build.max() + 1000, size=3_000_001)
+    probe[::2] = build[rng.integers(0, n, size=len(probe[::2]))]
+    if kind.endswith("int32"):
+        build, probe = build.astype(np.int32), probe.astype(np.int32)
+    check_join(ctx, stream, build, rng.integers(-2**40, 2**40, size=n), probe)
+
+
+@pytest.mark.parametrize("shuffled", [False, True])
+@pytest.mark.parametrize("cap", [1000, 2_999_999])
+def test_small_output_at_millions_of_probes(ctx, stream, shuffled, cap):
+    n = 1_100_000
+    rng = np.random.default_rng(3)
+    build = np.arange(n) * 4 + rng.integers(0, 4, size=n)
+    probe = np.repeat(build, 3)[:3_000_000]
+    if shuffled:
+        rng.shuffle(build)
+    check_join(ctx, stream, build, np.arange(n), probe, cap=cap)
+
+
+def test_even_keys_with_strays(ctx, stream):
+    """Keys far outside the sampled range, negative and positive, among even
+    ones; probes that miss on both sides."""
+    n = 2_000_000
+    rng = np.random.default_rng(4)
+    build = np.arange(n) * 8 + rng.integers(0, 8, size=n)
+    at = rng.choice(np.setdiff1d(np.arange(1, n - 1), np.round(np.linspace(0, n - 1, 512))),
+                    200, replace=False)
+    build[at[:100]] = -2**62 - np.arange(100)
+    build[at[100:]] = 2**62 + np.arange(100)
+    probe = np.concatenate([build, build + 1, [-2**63 + 1, 2**63 - 1, 2**62 + 50]])
+    check_join(ctx, stream, build, np.arange(n), probe)
