@@ -528,9 +528,11 @@ constexpr int kSub = 2048;
 constexpr int kSubWarpRows = kSub / 8;     // rows of a warp in a sub-tile
 constexpr int kSubSteps = kSubWarpRows / 32;
 
-// The part of the bucket number that a pass orders by: `bits` bits from
-// `shift` on of a number of log2P bits (all of it, or half of it in a partition
-// in two passes).  One multiply, shift and mask per key.
+// What a pass orders by: the whole bucket number of log2P bits, or (PART, a
+// partition in two passes) `bits` bits of it from `shift` on.  One multiply and
+// shift per key, and a mask for a part: 4-byte rows are bound by instructions,
+// and a mask on the whole number cost them 2 %.
+template <bool PART>
 struct Digit {
   int log2P, bits, rshift;
   u32 mask;
@@ -540,6 +542,7 @@ struct Digit {
         mask((1u << bits_) - 1u) {}
   __host__ __device__ int count() const { return 1 << bits; }
   __device__ __forceinline__ u32 operator()(i64 k) const {
+    if constexpr (!PART) return fib_bucket(k, log2P);
     return (u32)(((u64)k * 0x9E3779B97F4A7C15ULL) >> rshift) & mask;
   }
 };
@@ -570,16 +573,16 @@ __host__ __device__ inline i64 chunk_begin(i64 n, i64 g, i64 k) {
 // Histogram of the scatter's chunks: hsplit blocks per chunk (chunk k =
 // blockIdx.x / hsplit), each counting a share of the chunk's rows and adding
 // its counts into hist[b * g + k] (zeroed before).
-template <typename T>
+template <typename T, bool PART, bool TOT>
 __global__ void __launch_bounds__(256, 8) k_part_hist_blk(const T* __restrict__ key, i64 n,
-                                                          Digit dg, u32* __restrict__ hist,
+                                                          Digit<PART> dg, u32* __restrict__ hist,
                                                           i64 g, int hsplit,
                                                           u64* __restrict__ tot) {
   extern __shared__ u32 sh[];
-  // With `tot` (the first of two passes) whole buckets are counted, into tot
-  // (over all rows: 64 bits) and, added up by digit, into hist.
-  const int P = tot ? 1 << dg.log2P : dg.count();
-  const Digit cd = tot ? Digit(dg.log2P, 0, dg.log2P) : dg;
+  // TOT (the first of two passes): whole buckets are counted, into tot (over
+  // all rows: 64 bits) and, added up by digit, into hist.
+  const int P = TOT ? 1 << dg.log2P : dg.count();
+  auto cd = [&](i64 k) { return TOT ? fib_bucket(k, dg.log2P) : dg(k); };
   for (int b = threadIdx.x; b < P; b += blockDim.x) sh[b] = 0;
   __syncthreads();
   const i64 k = blockIdx.x / hsplit, h = blockIdx.x % hsplit;
@@ -611,7 +614,7 @@ __global__ void __launch_bounds__(256, 8) k_part_hist_blk(const T* __restrict__ 
   for (i64 i = r0 + steps * kRows + threadIdx.x; i < r1; i += blockDim.x)
     atomicAdd(&sh[cd((i64)__ldg(key + i))], 1u);
   __syncthreads();
-  if (!tot) {
+  if (!TOT) {
     for (int b = threadIdx.x; b < P; b += blockDim.x)
       if (sh[b]) atomicAdd(&hist[(i64)b * g + k], sh[b]);
     return;
@@ -697,9 +700,9 @@ __device__ __forceinline__ void stage_column(const V* __restrict__ src, V* __res
   __syncthreads();
 }
 
-template <typename T>
+template <typename T, bool PART>
 __global__ void __launch_bounds__(256) k_part_scatter_blk(const T* __restrict__ key, i64 n,
-                                                          Digit dg, const i64* __restrict__ gofs,
+                                                          Digit<PART> dg, const i64* __restrict__ gofs,
                                                           PayArgs pa, T* __restrict__ out_key,
                                                           i64* d_offsets) {
   extern __shared__ __align__(16) unsigned char smem[];
@@ -846,10 +849,14 @@ __device__ __forceinline__ void gather_column(const char* buf, int off, V* __res
     if (j * 256 + (int)threadIdx.x < cnt) __stcs(dst + drow[j], col[src[j]]);
 }
 
-// (Three blocks per SM, as the buffers allow: left alone, the compiler holds it
-// to 40 registers with a spill, 5 % slower in two passes.)
-template <typename T, int SUB>
-__global__ void __launch_bounds__(256, 3) k_part_scatter_tma(i64 n, Digit dg,
+// BLOCKS: the launch bound.  Three blocks per SM (71 to 80 registers) where the
+// buffers leave room for three at most; rows of up to 9 bytes, of which more
+// blocks fit, take no bound: the compiler then holds the kernel to 40
+// registers.  60M rows of 8 bytes by 64: 443 us with room for three blocks, 450
+// us bounded to five (48 registers), 422 us with none; of 21 bytes by 32 587 us
+// with room for three and 629 us with none.
+template <typename T, bool PART, int SUB, int BLOCKS>
+__global__ void __launch_bounds__(256, BLOCKS) k_part_scatter_tma(i64 n, Digit<PART> dg,
                                                           const i64* __restrict__ gofs,
                                                           TmaCols tc, i64* d_offsets,
                                                           i64 spin_limit, DevStatus* st) {
@@ -2152,30 +2159,11 @@ pq_status pq_filter(pq_ctx* ctx, pq_col col, int op, int64_t c, const int64_t* s
 }  // extern "C"
 
 namespace {
-// Blocks of a scatter kernel resident per SM with `smem` bytes of dynamic
-// shared memory; what does not depend on smem is asked of the runtime once per
-// device (two threads that ask at once find the same).
-template <auto K>
-int part_blocks(int device, size_t smem) {
-  static std::atomic<int> known[64];
-  std::atomic<int>* const at = device >= 0 && device < 64 ? &known[device] : nullptr;
-  int most = at ? at->load(std::memory_order_acquire) : 0;
-  if (!most) {
-    if (cudaFuncSetAttribute((const void*)K, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             200 * 1024) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&most, (const void*)K, 256, 0) != cudaSuccess)
-      cudaGetLastError();
-    most = std::max(most, 1);
-    if (at) at->store(most, std::memory_order_release);
-  }
-  constexpr size_t kPerSm = 228 * 1024, kPerBlock = 1024 + 256;  // reserved and static, per block
-  return std::max(1, std::min(most, (int)(kPerSm / (smem + kPerBlock))));
-}
-
 // One stable pass of the partition: rows ordered by digit `dg` of their
 // bucket.  d_offsets: the digits' offsets (or null); tot: null, or counts of
 // whole buckets to be added to (zeroed by the caller).
-pq_status part_pass(pq_ctx* ctx, pq_col key, const pq_col* payload, int npay, Digit dg,
+template <bool PART>
+pq_status part_pass(pq_ctx* ctx, pq_col key, const pq_col* payload, int npay, Digit<PART> dg,
                     void* out_key, void* const* out_payload, i64* d_offsets, u64* tot,
                     cudaStream_t s) {
   const i64 n = key.n;
@@ -2202,30 +2190,31 @@ pq_status part_pass(pq_ctx* ctx, pq_col key, const pq_col* payload, int npay, Di
     tc.es[1 + j] = (int)pqh::dtype_size(payload[j].type);
     aligned = aligned && ((uintptr_t)payload[j].data & 15) == 0;
   }
-  // Sub-tiles of 4096 rows from 512 buckets on (when they fit; of narrow rows
-  // from 256 on), so that a bucket's run in a sub-tile fills its sectors; 2048
-  // otherwise.
-  auto layout = [&](int sub) {
+  // Sub-tiles of 4096 rows from 512 buckets on (when they fit; of 5 to 8 bytes a
+  // row from 256 on), so that a bucket's run in a sub-tile fills its sectors;
+  // 2048 otherwise.  By 256, 60M rows of 8 bytes: 565 -> 445 us, of 4 bytes 460
+  // -> 468; 4M of 8 bytes 70 -> 73.
+  auto layout = [&](int rows) {
     int off = 0;
-    for (int c = 0; c < tc.n; ++c) tc.off[c] = off, off += sub * tc.es[c];
+    for (int c = 0; c < tc.n; ++c) tc.off[c] = off, off += rows * tc.es[c];
     tc.buf_bytes = off;
-    return tma_smem(P, tc.buf_bytes, sub);
+    return tma_smem(P, tc.buf_bytes, rows);
   };
   int sub = 4096;
-  size_t smem_tma = layout(sub);
-  if (dg.bits < 8 || (dg.bits == 8 && tc.buf_bytes > 32 * 1024) || smem_tma > 200 * 1024)
-    smem_tma = layout(sub = kSub);
-  const bool use_tma = aligned && smem_tma <= 200 * 1024;
-  const size_t smem = use_tma ? smem_tma : staged_smem(P);
-  const i64 rows_sub = use_tma ? sub : kSub;
-  int occ = 1;
-  PQ_DISPATCH_T(key.type, T, {
-    occ = !use_tma      ? part_blocks<k_part_scatter_blk<T>>(ctx->device, smem)
-          : sub == 4096 ? part_blocks<k_part_scatter_tma<T, 4096>>(ctx->device, smem)
-                        : part_blocks<k_part_scatter_tma<T, kSub>>(ctx->device, smem);
-  });
-  const i64 g = std::max<i64>(1, std::min<i64>((n + rows_sub - 1) / rows_sub,
-                                               (i64)ctx->num_sms * occ));
+  size_t smem = layout(sub);
+  const int row_bytes = tc.buf_bytes / sub;
+  const bool runs = dg.bits >= 9 || (dg.bits == 8 && row_bytes > 4 && row_bytes <= 8);
+  if (!runs || smem > 200 * 1024) smem = layout(sub = kSub);
+  const bool use_tma = aligned && smem <= 200 * 1024;
+  if (!use_tma) sub = kSub, smem = staged_smem(P);
+  // Blocks per SM: by shared memory (228 KB, 1 KB and the static part of it
+  // taken per block) and, at most, by registers.
+  // 9-byte rows, of which four blocks fit, gain by them up to 64 buckets (60M by
+  // 32: 447 us at four, 463 at three; by 128 607 and 560).
+  i64 occ = std::max<i64>(1, std::min<i64>(use_tma ? 5 : 6, 228 * 1024 / (i64)(smem + 1024 + 256)));
+  const bool bound = PART || sub == 4096 || occ <= 3 || (occ == 4 && dg.bits >= 7);
+  if (use_tma && bound) occ = std::min<i64>(occ, 3);
+  const i64 g = std::max<i64>(1, std::min<i64>((n + sub - 1) / sub, (i64)ctx->num_sms * occ));
   const i64 m = g * P;
   const i64 stiles = (m + 4095) / 4096;
   // One block of scratch: the scan's state and the histogram (both zeroed),
@@ -2244,25 +2233,36 @@ pq_status part_pass(pq_ctx* ctx, pq_col key, const pq_col* payload, int npay, Di
   const int hsplit = tot ? 1 : (int)std::max<i64>(
       1, std::min<i64>(((i64)ctx->num_sms * 8) / g, (n / g) / 4096));
   PQ_DISPATCH_T(key.type, T, {
-    k_part_hist_blk<T><<<(unsigned)(g * hsplit), 256, (size_t)(tot ? 1 << dg.log2P : P) * 4, s>>>(
-        (const T*)key.data, n, dg, hist, g, hsplit, tot);
+    const size_t hist_smem = (size_t)(tot ? 1 << dg.log2P : P) * 4;
+    auto count = [&](auto k) {
+      k<<<(unsigned)(g * hsplit), 256, hist_smem, s>>>((const T*)key.data, n, dg, hist, g, hsplit,
+                                                       tot);
+    };
+    if constexpr (PART) tot ? count(k_part_hist_blk<T, PART, true>) : count(k_part_hist_blk<T, PART, false>);
+    else count(k_part_hist_blk<T, PART, false>);
     PQ_LAUNCHED(ctx);
     k_scan_u32<<<(unsigned)std::min<i64>(stiles, (i64)ctx->num_sms * 4), 256, 0, s>>>(
         hist, m, gofs, (u64*)(w + 256), (u32*)w, ctx->opt.spin_limit, ctx->d_status);
     PQ_LAUNCHED(ctx);
-    auto tma = [&](auto k) {
-      k<<<(unsigned)g, 256, smem, s>>>(n, dg, gofs, tc, d_offsets, ctx->opt.spin_limit,
-                                       ctx->d_status);
+    auto launch = [&](auto k, auto... args) -> pq_status {
+      PQ_CUDA(ctx, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+      k<<<(unsigned)g, 256, smem, s>>>(args...);
+      PQ_LAUNCHED(ctx);
+      return PQ_OK;
     };
     if (!use_tma)
-      k_part_scatter_blk<T><<<(unsigned)g, 256, smem, s>>>((const T*)key.data, n, dg, gofs, pa,
-                                                           (T*)out_key, d_offsets);
-    else if (sub == 4096)
-      tma(k_part_scatter_tma<T, 4096>);
-    else
-      tma(k_part_scatter_tma<T, kSub>);
+      return launch(k_part_scatter_blk<T, PART>, (const T*)key.data, n, dg, (const i64*)gofs, pa,
+                    (T*)out_key, d_offsets);
+    auto scatter = [&](auto k) {
+      return launch(k, n, dg, (const i64*)gofs, tc, d_offsets, (i64)ctx->opt.spin_limit,
+                    ctx->d_status);
+    };
+    if constexpr (!PART) {  // a part has 64 digits at most
+      if (sub == 4096) return scatter(k_part_scatter_tma<T, PART, 4096, 3>);
+      if (!bound) return scatter(k_part_scatter_tma<T, PART, kSub, 0>);
+    }
+    return scatter(k_part_scatter_tma<T, PART, kSub, 3>);
   });
-  PQ_LAUNCHED(ctx);
   return PQ_OK;
 }
 
@@ -2339,10 +2339,10 @@ pq_status pq_partition(pq_ctx* ctx, pq_col key, const pq_col* payload, int npay,
       void* o1[PQ_MAX_PAYLOAD];
       k1.data = w + at[0];
       for (int j = 0; j < npay; ++j) p1[j] = payload[j], p1[j].data = o1[j] = w + at[1 + j];
-      pq_status st = part_pass(ctx, key, payload, npay, Digit(log2P, 0, lo), w + at[0], o1, nullptr,
+      pq_status st = part_pass(ctx, key, payload, npay, Digit<true>(log2P, 0, lo), w + at[0], o1, nullptr,
                                tot, s);
       if (st == PQ_OK)
-        st = part_pass(ctx, k1, p1, npay, Digit(log2P, lo, log2P - lo), out_key, out_payload,
+        st = part_pass(ctx, k1, p1, npay, Digit<true>(log2P, lo, log2P - lo), out_key, out_payload,
                        nullptr, nullptr, s);
       if (st == PQ_OK) {
         k_part_offsets<<<1, 1024, 0, s>>>(tot, P, n, (i64*)d_offsets);
@@ -2353,7 +2353,7 @@ pq_status pq_partition(pq_ctx* ctx, pq_col key, const pq_col* payload, int npay,
     }
   }
   if (log2P <= kStagedMaxLog2)
-    return part_pass(ctx, key, payload, npay, Digit(log2P, 0, log2P), out_key, out_payload,
+    return part_pass(ctx, key, payload, npay, Digit<false>(log2P, 0, log2P), out_key, out_payload,
                      (i64*)d_offsets, nullptr, s);
   const i64 ntiles = (n + kPartTile - 1) / kPartTile;
   const i64 m = ntiles * P;
