@@ -1819,6 +1819,10 @@ __global__ void __launch_bounds__(256) k_gb_emit(const longlong2* __restrict__ t
 }
 
 // ================================================================ top-k ====
+// Least pairs of a block beyond 2048 in all.  3.1M of 12.5M groups over a sum,
+// found by an aggregate-first plan of 50M rows: the plan takes 353 us with 1024,
+// 359 us with 256 or 2048; 250k groups, k = 64: 214, 220 and 205 us.
+constexpr int kTopkPer = 1024;
 __global__ void __launch_bounds__(256, 2) k_topk(const i64* __restrict__ keys,
                                               const i64* __restrict__ sums, i64 n_cap,
                                               const i64* d_n, int K, i64* part_k, i64* part_s,
@@ -1832,10 +1836,10 @@ __global__ void __launch_bounds__(256, 2) k_topk(const i64* __restrict__ keys,
   __shared__ LaneRankSmem<256> s_lr;
   chain_begin();
   const i64 n = d_n ? min(*d_n, n_cap) : n_cap;
-  // Only the first nb blocks take pairs (at least 2048 each: eight per thread),
-  // so that a small count read on the device leaves few lists to merge, or
-  // none.
-  const int nb = (int)max((i64)1, min((i64)gridDim.x, (n + 2047) / 2048));
+  // Only the first nb blocks take pairs, so that a small count read on the
+  // device leaves few lists to merge, or none: one block up to 2048 pairs, else
+  // at least kTopkPer each.
+  const int nb = n <= 2048 ? 1 : (int)min((i64)gridDim.x, (n + kTopkPer - 1) / kTopkPer);
   if ((int)blockIdx.x >= nb) return;  // no pairs: the nb blocks take the ticket
   const i64 per = (n + nb - 1) / nb;
   const i64 lo = min(n, per * blockIdx.x), hi = min(n, lo + per);
@@ -1849,28 +1853,33 @@ __global__ void __launch_bounds__(256, 2) k_topk(const i64* __restrict__ keys,
   // are merged in shared memory (TopList).
   int cnt = -1;
   if (K <= 32) {
-    // A first threshold: the K-th best of the threads' best sums among 16 of
-    // their pairs, spread over their shares (a sorted input then gives a
-    // threshold near its end).  At least K pairs are not below it, so a pair
-    // below it cannot be among the block's K best: only the others enter the
-    // lists, which keeps the lanes of a warp on the same path.  Blocks with
-    // fewer than 16 pairs per thread skip it (block-uniform).
+    // A first threshold: the K-th best of the threads' best pairs, each of 16
+    // spread over the thread's share (a sorted input then gives a threshold
+    // near its end).  At least K pairs are not after it, so a pair after it
+    // cannot be among the block's K best: only the others enter the lists,
+    // which keeps the lanes of a warp on the same path.  Blocks with fewer than
+    // 16 pairs per thread skip it (block-uniform).
     bool filt = false;
-    i64 ths = 0;
+    i64 thk = 0, ths = 0;
     if (hi - lo >= 16 * 256) {
       const i64 mine = (hi - lo - threadIdx.x + 255) / 256;  // 16 at least
+      const i64 at = lo + threadIdx.x;
       i64 x[16];
 #pragma unroll
-      for (int q = 0; q < 16; ++q) x[q] = __ldcs(sums + lo + threadIdx.x + mine * q / 16 * 256);
-      i64 hs = x[0];
+      for (int q = 0; q < 16; ++q) x[q] = __ldcs(sums + at + mine * q / 16 * 256);
+      i64 hs = x[0], hk = INT64_MAX;
 #pragma unroll
       for (int q = 1; q < 16; ++q) hs = max(hs, x[q]);
-      s_lr.hk[threadIdx.x] = 0, s_lr.hs[threadIdx.x] = hs;
+#pragma unroll
+      for (int q = 0; q < 16; ++q)
+        if (x[q] == hs) hk = min(hk, __ldcs(keys + at + mine * q / 16 * 256));
+      s_lr.hk[threadIdx.x] = hk, s_lr.hs[threadIdx.x] = hs;
       __syncthreads();
-      if (rank_among(s_lr.hk, s_lr.hs, 256, 0, hs, (int)threadIdx.x) == K - 1) s_lr.ths = hs;
+      if (rank_among(s_lr.hk, s_lr.hs, 256, hk, hs, (int)threadIdx.x) == K - 1)
+        s_lr.thk = hk, s_lr.ths = hs;
       __syncthreads();
       filt = true;
-      ths = s_lr.ths;
+      thk = s_lr.thk, ths = s_lr.ths;
       __syncthreads();  // tk_lane_rank reuses s_lr
     }
     LaneTop T;
@@ -1878,14 +1887,23 @@ __global__ void __launch_bounds__(256, 2) k_topk(const i64* __restrict__ keys,
     i64 i = lo + threadIdx.x;
     if (filt) {
       // Most pairs fall short by their sum alone: only the sums are read, 16
-      // in flight, and the key of the few that pass (so half the bytes).
+      // in flight, and the keys of those that pass or tie (so half the bytes).
+      // Without the keys of ties all of 15M equal sums entered the lists: 168 us
+      // instead of 66 (with them 15M sums that differ take 51 us, 47 without).
       for (; i + 15 * 256 < hi; i += 16 * 256) {
         i64 s[16];
 #pragma unroll
         for (int u = 0; u < 16; ++u) s[u] = __ldcs(sums + i + u * 256);
-        u32 m = 0;
+        u32 m = 0, tie = 0;
 #pragma unroll
-        for (int u = 0; u < 16; ++u) m |= (u32)(s[u] >= ths) << u;
+        for (int u = 0; u < 16; ++u) m |= (u32)(s[u] > ths) << u, tie |= (u32)(s[u] == ths) << u;
+        if (tie) {
+#pragma unroll
+          for (int u = 0; u < 16; ++u)
+            s[u] = (tie >> u) & 1u ? __ldcs(keys + i + u * 256) : INT64_MAX;
+#pragma unroll
+          for (int u = 0; u < 16; ++u) m |= (tie >> u & (u32)(s[u] <= thk)) << u;
+        }
         for (; m; m &= m - 1) {
           const i64 e = i + (__ffs(m) - 1) * 256;
           T.insert(keys[e], sums[e]);
@@ -1902,7 +1920,7 @@ __global__ void __launch_bounds__(256, 2) k_topk(const i64* __restrict__ keys,
     }
     for (; i < hi; i += blockDim.x) {
       const i64 xk = keys[i], xs = sums[i];
-      if (!filt || xs >= ths) T.insert(xk, xs);
+      if (!filt || xs > ths || (xs == ths && xk <= thk)) T.insert(xk, xs);
     }
     cnt = tk_lane_rank(T, K, s_lr, bk, bs);
   }
