@@ -54,7 +54,8 @@ struct QCtr {
   u64 d_nmin, d_umax, m_nmin, m_umax;
   u64 m_umin;  // M bitmap: ukey of bit 0
   u64 m_bits;  // M bitmap: bit count (0 = no bitmap)
-  u64 pad[2];
+  u64 m_copies;  // dense M dictionary: most members of one key (the copy count)
+  u64 pad;
   // Regions the D and M fills clear: byte offset from the table's start and
   // 16-byte units (set by the scans' last blocks).
   u64 d_fill_off, d_fill_units, m_fill_off, m_fill_units;
@@ -1449,7 +1450,9 @@ __global__ void __launch_bounds__(256) k_plan_mrank(Batch b) {
 }
 
 // Copies per key when the members repeat keys: count the members of each
-// dense slot (the F probe multiplies a row's revenue by it).  With a key list
+// dense slot (the F probe multiplies a row's revenue by it), and the most of
+// any (fast_commit's bound: with the number of M rows in its place, one key
+// held twice sent 1M F rows to the checked additions).  With a key list
 // (tiles of 128 entries) the keys come from it; with a static bitmap (tiles
 // of M rows) the M rows are tested again (date, D-set) for their members.
 __global__ void __launch_bounds__(256) k_plan_mdup(Batch b) {
@@ -1489,28 +1492,53 @@ __global__ void __launch_bounds__(256) k_plan_mdup(Batch b) {
     u32* cnt = reinterpret_cast<u32*>(reinterpret_cast<char*>(q.ht_tag) +
                                       dense_layout(n, q.ctr->m_bits).cnt);
     const u64 umin = q.ctr->m_umin;
+    u32 most = 0;  // copies of a key seen by this lane
+    auto report = [&]() {
+      most = __reduce_max_sync(kFull, most);
+      if (lane == 0 && most > ld_volatile_u64(&q.ctr->m_copies))
+        atomicMax((unsigned long long*)&q.ctr->m_copies, (unsigned long long)most);
+    };
     if (q.m_static) {
       const TableView dt = table_view(q.dset_tag, *q.dset_log2, false);
       const u64* dhdr = reinterpret_cast<const u64*>(q.dset_log2);
       const u64 d_umin = dhdr[1], d_bits = dhdr[2];
       const i64 r0 = (t - pre[qi]) * q.m_tile, r1 = min(q.n_m, r0 + q.m_tile);
-      for (i64 r = r0 + lane; r < r1; r += 32) {
-        if (!pass(q.pm, __ldg(q.m_date + r))) continue;
-        const i64 dr = __ldg(q.m_dref + r);
-        const u64 di = ukey(dr) - d_umin;
-        const bool mem = d_bits ? di < d_bits && bit_test(dt.keybm, di, keep)
-                                : set_contains(dt, dr, keep);
-        const u64 idx = mem ? ukey(__ldg(q.m_key + r)) - umin : ~0ULL;
-        if (idx < q.m_sb) atomicAdd(cnt + dense_rank(dv, idx, keep), 1u);
+      // Four rows per lane side by side: each is a chain of six waits.
+      constexpr int kR = 4;
+      for (i64 rb = r0; rb < r1; rb += 32 * kR) {
+        u64 idx[kR];
+        u32 was[kR];
+#pragma unroll
+        for (int j = 0; j < kR; ++j) {
+          const i64 r = rb + 32 * j + lane;
+          idx[j] = r < r1 && pass(q.pm, __ldg(q.m_date + r)) ? (u64)r : ~0ULL;
+        }
+#pragma unroll
+        for (int j = 0; j < kR; ++j) {
+          if (idx[j] == ~0ULL) continue;
+          const i64 r = (i64)idx[j], dr = __ldg(q.m_dref + r);
+          const u64 di = ukey(dr) - d_umin;
+          const bool mem = d_bits ? di < d_bits && bit_test(dt.keybm, di, keep)
+                                  : set_contains(dt, dr, keep);
+          idx[j] = mem ? ukey(__ldg(q.m_key + r)) - umin : ~0ULL;
+        }
+#pragma unroll
+        for (int j = 0; j < kR; ++j)
+          was[j] = idx[j] < q.m_sb ? atomicAdd(cnt + dense_rank(dv, idx[j], keep), 1u) + 1 : 0u;
+#pragma unroll
+        for (int j = 0; j < kR; ++j) most = max(most, was[j]);
       }
+      report();
       continue;
     }
     const i64 i0 = (t - pre[qi]) * kTB;
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       const i64 idx = i0 + j * 32 + lane;
-      if (idx < n) atomicAdd(cnt + dense_rank(dv, ukey(q.mlist[idx]) - umin, keep), 1u);
+      if (idx < n)
+        most = max(most, atomicAdd(cnt + dense_rank(dv, ukey(q.mlist[idx]) - umin, keep), 1u) + 1);
     }
+    report();
   }
   finish(b.work, kPhMdup);
 }
@@ -1535,9 +1563,11 @@ struct ProbeCtx {
 // The fast commit of a plan (see PlanDev::rev_max), for `hits` hits.
 __device__ __forceinline__ bool fast_commit(const PlanDev& q, u64 hits) {
   if (!q.rev_max) return false;
-  // Largest multiplicity: 1 for a dense dictionary of distinct keys, else
-  // the plan's M rows (a hash table may hold a key in many slots).
-  const unsigned __int128 mult = q.ctr->m_bits && !q.ctr->dup ? 1 : (u64)max(q.n_m, (i64)1);
+  // Largest multiplicity: 1 for a dense dictionary of distinct keys, the
+  // measured one if keys repeat, else the plan's M rows (a hash table may hold
+  // a key in many slots).
+  const unsigned __int128 mult = !q.ctr->m_bits ? (u64)max(q.n_m, (i64)1)
+                                 : q.ctr->dup   ? max(q.ctr->m_copies, (u64)1) : 1;
   return (unsigned __int128)hits * q.rev_max * mult < ((unsigned __int128)1 << 63);
 }
 __device__ __forceinline__ void red_add(i64* p, i64 v) {
@@ -1989,8 +2019,12 @@ __global__ void __launch_bounds__(256, 4) k_plan_fscan(Batch b) {
 // one reduction, or an addition in the block's table of frequent groups.  The
 // first-hit bit is set only by a row whose revenue is not positive: any other
 // group is known by its sum, which is then not zero (the top-k pass reads the
-// sums of all slots).  Where a sum might leave int64 (fast_commit does not
-// hold), each addition is checked and every row sets its bit.
+// sums of all slots).  Where a sum might leave int64 (repeated M keys, so that
+// fast_commit does not hold, or very large prices),
+// rows that join commit as in the probe: equal groups of 32 such rows are
+// summed in 128 bits, frequent ones in the block's shared table, with every
+// addition checked.  (Each row adding by itself: 20M Zipf rows, one M key held twice,
+// 779 -> 1698 us.)
 // A warp takes steps of 128 rows (lane l: rows 4l .. 4l+3), the grid's warps
 // consecutive ones; date is read two steps ahead, the other columns one.
 // What bounds it is random access: two per row (the record, the sum), where
@@ -2002,15 +2036,22 @@ __global__ void __launch_bounds__(256, 4) k_plan_fscan(Batch b) {
 // takes a reduction per 1.8 ns) 26 ms; of 4096 entries, which leave the L1
 // less room for the records, 4.4 ms.
 constexpr int kHotLog2 = 10;
-template <bool VEC>
-__device__ __forceinline__ void fdirect(const Batch& b, HotSums<kHotLog2>& hot) {
+template <bool VEC, bool exact>
+__device__ __forceinline__ void fdirect(const Batch& b, HotSums<kHotLog2>& hot, u64* akey,
+                                        i64* asum, i64* sc) {
   const PlanDev& q = b.q[0];
   QCtr* const c = q.ctr;
-  hot.clear();
-  __syncthreads();
   const int lane = threadIdx.x & 31;
   const u64 keep = policy_keep(), strm = policy_stream();
   const i64 n = q.n_f;
+  if (!exact) hot.clear();
+  __syncthreads();
+  // Checked additions use the table's place for a ring of rows per warp.
+  constexpr u32 kRing = 31 + 64;
+  static_assert(8 * (kRing * 12 + 8) <= sizeof(hot), "ring");
+  i64* const rval = reinterpret_cast<i64*>(&hot) + (threadIdx.x >> 5) * (kRing * 12 / 8 + 1);
+  u32* const rslot = reinterpret_cast<u32*>(rval + kRing);
+  u32 nring = 0;
   const i64* const mkey = q.f_mkey;
   const i64* const price = q.f_price;
   const signed char* const disc = q.f_disc;
@@ -2023,7 +2064,7 @@ __device__ __forceinline__ void fdirect(const Batch& b, HotSums<kHotLog2>& hot) 
   u32* const hit = reinterpret_cast<u32*>(gb + L.hit);
   i64* const sums = reinterpret_cast<i64*>(gb + L.sums);
   const u32* const cnt = c->dup ? reinterpret_cast<const u32*>(gb + L.cnt) : nullptr;
-  const bool exact = !fast_commit(q, (u64)n);
+  const GroupStore g = {hit, sums, 1};
   const i64 steps = (n + 127) / 128, stride = (i64)gridDim.x * (blockDim.x >> 5);
   const i64 s0 = (i64)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   auto ld_d = [&](i64 s) -> int4 {
@@ -2087,18 +2128,37 @@ __device__ __forceinline__ void fdirect(const Batch& b, HotSums<kHotLog2>& hot) 
     }
     hits += __popc(live);
     if (exact) {
+      // Into the warp's ring in row order, half a warp's rows at a time, and
+      // from there 32 at a time as the probe commits hits.
+      const u32 mine = __popc(live);
+      u32 incl = mine;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const u32 y = __shfl_up_sync(kFull, incl, o);
+        if (lane >= o) incl += y;
+      }
+      const u32 half = __shfl_sync(kFull, incl, 15), all = __shfl_sync(kFull, incl, 31);
 #pragma unroll 1
-      for (int j = 0; j < 4; ++j) {
-        if (!((live >> j) & 1u)) continue;
-        const i64 pj = j == 0 ? pA[0] : j == 1 ? pA[1] : j == 2 ? pA[2] : pA[3];
-        const u32 sj = j == 0 ? slot[0] : j == 1 ? slot[1] : j == 2 ? slot[2] : slot[3];
-        const __int128 v128 = (__int128)(cnt ? (i64)__ldg(cnt + sj) : 1) *
-                              ((__int128)pj * (100 - (i64)(signed char)(dA >> (8 * j))));
-        const i64 vj = (i64)v128;
-        red_or(hit + (sj >> 5), 1u << (sj & 31));
-        const i64 old = (i64)atomicAdd((u64*)(sums + sj), (u64)vj);
-        if (v128 != (__int128)vj || add_overflows(old, vj))
-          q_latch(c, b.st, PQ_ERR_OVERFLOW, (i64)sj);
+      for (int h = 0; h < 2; ++h) {
+        u32 at = nring + incl - mine - (h ? half : 0u);
+        if ((lane >> 4) == h) {
+#pragma unroll 1
+          for (int j = 0; j < 4; ++j) {
+            if (!((live >> j) & 1u)) continue;
+            const i64 pj = j == 0 ? pA[0] : j == 1 ? pA[1] : j == 2 ? pA[2] : pA[3];
+            const u32 sj = j == 0 ? slot[0] : j == 1 ? slot[1] : j == 2 ? slot[2] : slot[3];
+            const __int128 v128 = (__int128)(cnt ? (i64)__ldg(cnt + sj) : 1) *
+                                  ((__int128)pj * (100 - (i64)(signed char)(dA >> (8 * j))));
+            if (v128 != (__int128)(i64)v128) q_latch(c, b.st, PQ_ERR_OVERFLOW, (i64)sj);
+            rslot[at] = sj, rval[at] = (i64)v128, ++at;
+          }
+        }
+        nring += h ? all - half : half;
+        __syncwarp();
+        for (; nring >= 32; nring -= 32)
+          commit_hits_g(b, sc, akey, asum, true, 0, rslot[nring - 32 + lane],
+                        rval[nring - 32 + lane], &g, true);
+        __syncwarp();
       }
     } else {
 #pragma unroll
@@ -2122,11 +2182,25 @@ __device__ __forceinline__ void fdirect(const Batch& b, HotSums<kHotLog2>& hot) 
 #pragma unroll
     for (int j = 0; j < 4; ++j) kA[j] = kB[j], pA[j] = pB[j];
   }
+  if (exact) {  // block-uniform
+    const bool act = (u32)lane < nring;
+    commit_hits_g(b, sc, akey, asum, act, 0, act ? rslot[lane] : 0u, act ? rval[lane] : 0, &g, true);
+  }
   __syncthreads();
-  for (int i = threadIdx.x; i < hot.kN; i += blockDim.x)
+  for (int i = threadIdx.x; !exact && i < hot.kN; i += blockDim.x)
     if (hot.key[i] != kHotFree) red_add(sums + hot.key[i], (i64)((u64)hot.hi[i] << 32 | hot.lo[i]));
   const u32 h = __reduce_add_sync(kFull, (u32)hits);  // a warp's rows: below 2^32
   if (lane == 0 && h) atomicAdd(&c->hits_total, (u64)h);
+}
+
+// With checked additions: a function of its own, as it is rare and would take
+// registers from the other one.  (The other one as a function: 40M rows that all
+// join 356 -> 411 us; inlined, the probe of a hit list takes as long as before
+// it was there, though the kernel spills.)
+template <bool VEC>
+__device__ __noinline__ void fdirect_checked(const Batch& b, HotSums<kHotLog2>& hot, u64* akey,
+                                             i64* asum, i64* sc) {
+  fdirect<VEC, true>(b, hot, akey, asum, sc);
 }
 
 // F probe: warp tiles of the hit list (hp_tile rows), 32 per batch: each
@@ -2136,7 +2210,7 @@ __device__ __forceinline__ void fdirect(const Batch& b, HotSums<kHotLog2>& hot) 
 // memory).  A plan with at least 2048 hits per block of the grid (skewed or
 // pass-all data, where groups repeat within a block) first tries the
 // block's shared aggregation table.
-__global__ void __launch_bounds__(256, 4) k_plan_fprobe(Batch b) {
+__global__ void __launch_bounds__(256, 4) k_plan_fprobe(const __grid_constant__ Batch b) {
   chain_begin();
   __shared__ u64 s_akey[kAgg];
   __shared__ i64 s_asum[kAgg];
@@ -2144,16 +2218,23 @@ __global__ void __launch_bounds__(256, 4) k_plan_fprobe(Batch b) {
   extern __shared__ __align__(16) unsigned char s_dyn[];  // only when direct_ok
   const i64* pre = b.dyn + 7 * (b.nq + 1);
   i64 total;
-  if (direct_verdict(b, pre + b.nq, total)) {
-    auto& hot = *reinterpret_cast<HotSums<kHotLog2>*>(s_dyn);
-    if (b.q[0].vec) fdirect<true>(b, hot);
-    else fdirect<false>(b, hot);
-  }
+  const bool direct = direct_verdict(b, pre + b.nq, total);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   i64* sc = s_sc[warp];
   for (int i = threadIdx.x; i < kAgg; i += blockDim.x) s_akey[i] = 0, s_asum[i] = 0;
   __syncthreads();
   const u64 agg_min = (u64)gridDim.x * 2048;
+  if (direct) {
+    auto& hot = *reinterpret_cast<HotSums<kHotLog2>*>(s_dyn);
+    u64* const akey = (u64)b.q[0].n_f >= agg_min ? s_akey : nullptr;
+    if (fast_commit(b.q[0], (u64)b.q[0].n_f)) {
+      if (b.q[0].vec) fdirect<true, false>(b, hot, akey, s_asum, sc);
+      else fdirect<false, false>(b, hot, akey, s_asum, sc);
+    } else {
+      if (b.q[0].vec) fdirect_checked<true>(b, hot, akey, s_asum, sc);
+      else fdirect_checked<false>(b, hot, akey, s_asum, sc);
+    }
+  }
   const u64 keep = policy_keep();
   const bool ov = b.ov.table == 3;
   WarpClaim wc;
