@@ -374,11 +374,11 @@ constexpr int kMaxPartLog2 = 10;
 constexpr int kPT = 2048;
 constexpr int kAT = 1024;
 
-// The direct F pass (fdirect) takes a plan whose members are at least
-// one M row in kDirectShare: then enough F rows join that reading price and
-// discount with the key costs less than a hit list written, read back and
-// probed in a kernel of its own (10M clustered rows, all joining: the plan
-// 314 -> 173 us; the 60M-row plan of which 0.5 % join stays at 259 us).
+// The direct F pass (fdirect) takes a plan of which enough F rows join that
+// reading price and discount with the key, and all sums in the top-k, costs less
+// than a hit list written, read back and probed in a kernel of its own.  Plans
+// whose members are less than one M row in kDirectShare are not looked at
+// further; for the others direct_vote samples F.
 constexpr i64 kDirectShare = 8;
 // The M scan's verdict (Batch::direct_ok plans): a word of the work area, so
 // that the later kernels know it after a single load.
@@ -842,14 +842,69 @@ __global__ void __launch_bounds__(256) k_plan_dbuild(Batch b) {
 }
 
 // ------------------------------------------------------------------ mscan ----
+// Whether the batch's only plan takes the direct F pass (the M scan's last
+// block of 8 warps, its bitmap set): 1024 rows spread over F give the share f
+// that passes the date test and the share that also joins (3 us, for plans that
+// get here).  In bytes of the columns' rate,
+// the pass costs price and discount of every sector with a passing row (four
+// such rows), the sums of all members in the top-k and 5 us of its own; a hit
+// saves 80.  Against the hit list, 40M rows over 10M M rows: 15 % of M and all
+// of F's dates, 344 -> 305 us clustered and 509 -> 393 us Zipf; half of the
+// dates 305 -> 320, a tenth 243 -> 295; 4M rows that all join 197 -> 123, a
+// quarter of them 123 -> 124, 3 % of them 98 -> 123.  A plan whose sums may leave
+// int64 even when no M key repeats keeps the hit list, whose probe combines
+// more rows before each checked addition.
+__device__ __noinline__ void direct_vote(const PlanDev* qp, u32* verdict) {
+  const PlanDev& q = *qp;
+  const i64 members = ld_count(&q.ctr->mcount), n = q.n_f;
+  __shared__ u32 s_n[2];
+  bool take = members > 0 && members >= q.n_m / kDirectShare &&
+              80 * n > 35000000 + 8 * members && q.rev_max &&
+              (unsigned __int128)(u64)n * q.rev_max < ((unsigned __int128)1 << 63);
+  if (take) {  // block-uniform
+    constexpr int kPer = 4;
+    if (threadIdx.x < 2) s_n[threadIdx.x] = 0;
+    __syncthreads();
+    // A warp's rows are 32 in a row (pages are what a sample costs), the 32
+    // places of the 8 warps spread evenly, each somewhere in its part of F.
+    const i64 part = n / (8 * kPer);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const Pred32 pf = to32(q.pf);
+    const u64 ubase = q.m_su ^ 0x8000000000000000ULL;
+    i64 key[kPer];
+    int date[kPer];
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) {
+      const u32 i = j * 8 + warp;
+      const i64 r = i * part + (i64)__umul64hi((u64)(i + 1) * 0x9E3779B97F4A7C15ULL, part - 32) + lane;
+      key[j] = __ldg(q.f_mkey + r), date[j] = __ldg(q.f_date + r);
+    }
+    u32 pass = 0, join = 0;
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) {
+      const u64 idx = (u64)key[j] - ubase;
+      const bool p = pass32(pf, date[j]), in = p && idx < q.m_sb;
+      const u32 w = in ? __ldcg(reinterpret_cast<const u32*>(q.ht_tag) + (idx >> 5)) : 0u;
+      pass += p, join += (w >> (idx & 31)) & 1u;
+    }
+    pass = __reduce_add_sync(kFull, pass), join = __reduce_add_sync(kFull, join);
+    if (lane == 0) atomicAdd(&s_n[0], pass), atomicAdd(&s_n[1], join);
+    __syncthreads();
+    constexpr float kAll = 1.0f / (256 * kPer);
+    const float rows = (float)n, f = s_n[0] * kAll, h = s_n[1] * kAll;
+    take = 80.0f * h * rows > 9.0f * rows * fminf(1.0f, 4.0f * f) + 8.0f * members + 3.5e7f;
+  }
+  if (threadIdx.x == 0) *verdict = take;
+}
+
 // The M scan's last block: the M side's layout per plan (static bitmap, or
 // sized from the members' count and key range) and the tile counts of the
 // phases that follow.
 __device__ void mscan_finish(const Batch& b) {
+  if (b.direct_ok) direct_vote(&b.q[0], b.work + kDirectWord);
   block_prefix(b.dyn + 2 * (b.nq + 1), b.nq, [&](int qi) -> i64 {
     const PlanDev& q = b.q[qi];
     if (q.m_static) {  // bitmap over the table's key range, set by this scan
-      if (b.direct_ok) b.work[kDirectWord] = ld_count(&q.ctr->mcount) >= q.n_m / kDirectShare;
       q.ctr->mlog2 = q.m_e;
       q.ctr->m_umin = q.m_su;
       q.ctr->m_bits = q.m_sb;
@@ -2020,7 +2075,7 @@ __global__ void __launch_bounds__(256, 4) k_plan_fscan(Batch b) {
 // first-hit bit is set only by a row whose revenue is not positive: any other
 // group is known by its sum, which is then not zero (the top-k pass reads the
 // sums of all slots).  Where a sum might leave int64 (repeated M keys, so that
-// fast_commit does not hold, or very large prices),
+// fast_commit does not hold; without them such a plan does not take the pass),
 // rows that join commit as in the probe: equal groups of 32 such rows are
 // summed in 128 bits, frequent ones in the block's shared table, with every
 // addition checked.  (Each row adding by itself: 20M Zipf rows, one M key held twice,
