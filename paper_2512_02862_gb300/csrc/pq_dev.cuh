@@ -431,10 +431,25 @@ struct HotSums {
       if (cur == kHotFree) cur = slot;
     }
     if (cur != slot) return false;
+    put(h, v);
+    return true;
+  }
+  // Adds a slot that has an entry, or (claim) can have one.
+  __device__ __forceinline__ bool add_if(u32 slot, i64 v, bool claim) {
+    const u32 h = (slot * 0x9E3779B1u) >> (32 - LOG2);
+    u32 cur = *(volatile const u32*)&key[h];
+    if (claim && cur == kHotFree) {
+      cur = atomicCAS(&key[h], kHotFree, slot);
+      if (cur == kHotFree) cur = slot;
+    }
+    if (cur != slot) return false;
+    put(h, v);
+    return true;
+  }
+  __device__ __forceinline__ void put(u32 h, i64 v) {
     const u32 a = (u32)(u64)v, old = atomicAdd(&lo[h], a);
     const u32 up = (u32)((u64)v >> 32) + (old + a < old ? 1u : 0u);
     if (up) atomicAdd(&hi[h], up);
-    return true;
   }
 };
 

@@ -1361,18 +1361,57 @@ struct GbSummary {
   i64 first;        // runs before the first descent (all of them: no descent)
   i64 descents;     // rows whose key is below the row's before
   u32 over;         // the hash table did not hold the groups
+  u32 top;          // rows of the most frequent key in a sample (0: fewer than kGbTopHot)
 };
 struct GbWarp {
   u32 runs, before, descents;  // of the warp's rows; before its first descent
   int joined;                  // its first row continues the run before it
 };
 
+// How often the most frequent key comes among 1024 rows spread over the input:
+// from kGbTopHot of them on the tables keep frequent groups per block.
+constexpr int kGbSample = 1024;
+constexpr u32 kGbTopHot = 4;
+template <typename TK>
+__device__ __forceinline__ void gb_sample(const TK* __restrict__ key, i64 n, GbSummary* sum) {
+  constexpr int kN = 2 * kGbSample;
+  __shared__ i64 s_key[kN];
+  __shared__ u32 s_cnt[kN], s_top;
+  i64 k[kGbSample / 256];
+#pragma unroll
+  for (int j = 0; j < kGbSample / 256; ++j)
+    k[j] = (i64)__ldg(key + n / kGbSample * (j * 256 + threadIdx.x));
+  for (int i = threadIdx.x; i < kN; i += 256) s_key[i] = kEmpty, s_cnt[i] = 0;
+  if (threadIdx.x == 0) s_top = 0;
+  __syncthreads();
+#pragma unroll
+  for (int j = 0; j < kGbSample / 256; ++j) {
+    if (k[j] == kEmpty) continue;
+    u32 at = (u32)slot_hash(k[j]) & (kN - 1);
+    for (;; at = (at + 1) & (kN - 1)) {  // half of the slots stay free
+      const i64 was = (i64)atomicCAS((unsigned long long*)&s_key[at], (unsigned long long)kEmpty,
+                                     (unsigned long long)k[j]);
+      if (was == kEmpty || was == k[j]) break;
+    }
+    const u32 c = atomicAdd(&s_cnt[at], 1u) + 1;
+    if (c >= kGbTopHot) atomicMax(&s_top, c);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) sum->top = s_top;
+}
+
+// (The first block samples the keys meanwhile.)
 template <typename TK, bool VEC>
 __global__ void __launch_bounds__(256, 6) k_gb_scan(const TK* __restrict__ key, i64 n,
                                                     GbWarp* __restrict__ wout, GbSummary* sum) {
+  if (blockIdx.x == 0) {
+    gb_sample(key, n, sum);
+    return;
+  }
   __shared__ u64 s_lo[8], s_hi[8];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const i64 steps = (n + 127) / 128, nw = (i64)gridDim.x * 8, gw = (i64)blockIdx.x * 8 + warp;
+  const i64 steps = (n + 127) / 128, nw = (i64)(gridDim.x - 1) * 8;
+  const i64 gw = (i64)(blockIdx.x - 1) * 8 + warp;
   const i64 t0 = filter_share(steps, nw, gw), t1 = filter_share(steps, nw, gw + 1);
   u32 starts = 0, desc = 0, before = 0;
   bool any_desc = false, joined = false;
@@ -1653,57 +1692,126 @@ __device__ __forceinline__ void gb_each_run(const TK* __restrict__ key, const TV
   }
 }
 
-// Both tables below keep a block's frequent groups in shared memory (a
-// reduction on one address takes 1.8 ns: a key that holds a sixteenth of 30M
-// rows took the dense path to 3.3 ms, the hash table to 2.7 ms).
-constexpr int kGbHotLog2 = 11;
+// Slots of the hash table: keys and sums in arrays of their own (STRIDE 1) while
+// they fit in L2, so that the sectors of the keys are only read once they are
+// filled; {key, sum} side by side (STRIDE 2), one sector per row, in tables
+// beyond it (kGbPairBytes).  40M rows: of 400000 groups 0.62 and 1.2 ms, of 10M
+// groups 2.7 and 2.1 ms, of 40M 4.5 and 3.6 ms.
+constexpr size_t kGbPairBytes = 128 << 20;
+struct GbTable {
+  i64 *keys, *sums;
+  int log2cap;
+};
 
-// Hash table of {key, sum} slots, one sector per run.  With `over`, a table
-// that fills up is given up instead of reported: a key that finds no slot
-// within kGbMaxProbes sets the flag, and the others stop looking a line (8
-// slots) further on, so that the whole pass costs no more than a few lines a
-// row.
+// Rows of no frequent key, or few rows: a lane takes a row (rows in flight are
+// what counts: four rows per lane one after another took 40M rows of 400000
+// groups 616 -> 860 us), equal keys of a warp are added first, and a key that
+// a warp meets twice goes to the block's small table of frequent groups, which
+// the others only look at.  With `over`, a table that fills up is given up instead of
+// reported: a key that finds no slot within kGbMaxProbes sets the flag, and the
+// others stop looking a line (8 slots) further on, so that the whole pass costs
+// no more than a few lines a row.
 constexpr u64 kGbMaxProbes = 1024;
-template <typename TK, typename TV, bool VEC>
+// A key's slot, inserted if need be; ~0: none (`over` is set or was).
+template <int STRIDE>
+__device__ __forceinline__ u64 gb_slot(const GbTable& t, i64 k, u64 mask, u64 limit, u32* over,
+                                       DevStatus* st) {
+  u64 s = slot_hash(k) & mask;
+  for (u64 probes = 0; probes <= limit; ++probes) {
+    i64 cur = t.keys[STRIDE * s];  // a stale free slot is seen by the CAS
+    if (cur == kEmpty)
+      cur = (i64)atomicCAS((u64*)&t.keys[STRIDE * s], (u64)kEmpty, (u64)k);
+    if (cur == kEmpty || cur == k) return s;
+    if (over && (probes & 7) == 7 && *(volatile u32*)over) return ~0ULL;
+    s = (s + 1) & mask;
+  }
+  if (over) *(volatile u32*)over = 1;
+  else latch(st, PQ_ERR_CAPACITY, -1);
+  return ~0ULL;
+}
+// Adds the block's frequent groups to the table.
+template <int STRIDE, int HOT>
+__device__ __forceinline__ void gb_flush(const HotSums<HOT>& hot, const GbTable& t) {
+  __syncthreads();
+  for (int i = threadIdx.x; i < hot.kN; i += blockDim.x)
+    if (hot.key[i] != kHotFree)
+      atomicAdd((u64*)&t.sums[STRIDE * (u64)hot.key[i]], (u64)hot.hi[i] << 32 | hot.lo[i]);
+}
+template <typename TK, typename TV, int STRIDE>
+__global__ void __launch_bounds__(256) k_gb_rows(const TK* __restrict__ key,
+                                                 const TV* __restrict__ val, i64 n, GbTable t,
+                                                 DevStatus* st, u32* over) {
+  __shared__ HotSums<8> hot;
+  hot.clear();
+  __syncthreads();
+  const u64 mask = (1ULL << t.log2cap) - 1;
+  const u64 limit = over ? min(mask, kGbMaxProbes - 1) : mask;
+  const bool use_hot = t.log2cap < 32;
+  const int lane = threadIdx.x & 31;
+  const i64 gw = ((i64)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const i64 nwarps = ((i64)gridDim.x * blockDim.x) >> 5;
+  bool gone = false;  // the table is given up
+  for (i64 wb = gw * 32; wb < n; wb += nwarps * 32) {
+    if (over && __any_sync(kFull, gone)) break;
+    const i64 i = wb + lane;
+    bool active = i < n;
+    const i64 k = active ? (i64)__ldg(key + i) : kEmpty;
+    i64 v = active ? (i64)__ldg(val + i) : 0;
+    if (active && k == kEmpty) {
+      latch(st, PQ_ERR_RESERVED_KEY, i);
+      active = false;
+    }
+    const u32 peers = __match_any_sync(kFull, (u64)k);
+    if (__any_sync(kFull, active && __popc(peers) > 1)) {
+      i64 agg = 0;
+      for (int src = 0; src < 32; ++src) {
+        const i64 x = __shfl_sync(kFull, v, src);
+        if ((peers >> src) & 1u) agg += x;
+      }
+      v = agg;
+    }
+    if (!active || lane != __ffs(peers) - 1) continue;
+    const u64 s = gb_slot<STRIDE>(t, k, mask, limit, over, st);
+    if (s == ~0ULL) {
+      gone = true;
+      continue;
+    }
+    if (!(use_hot && hot.add_if((u32)s, v, __popc(peers) > 1)))
+      atomicAdd((u64*)&t.sums[STRIDE * s], (u64)v);
+  }
+  gb_flush<STRIDE>(hot, t);
+}
+
+// Many rows with frequent keys: runs as in the slot array below, and a large
+// table of frequent groups per block (a reduction on one address takes 1.8 ns:
+// a key that holds a sixteenth of 30M rows took the hash table to 2.7 ms and
+// the slot array to 3.3 ms).
+constexpr int kGbHotLog2 = 11;
+template <typename TK, typename TV, bool VEC, int STRIDE>
 __global__ void __launch_bounds__(256) k_gb_insert(const TK* __restrict__ key,
-                                                   const TV* __restrict__ val, i64 n,
-                                                   i64* __restrict__ slots, int log2cap,
+                                                   const TV* __restrict__ val, i64 n, GbTable t,
                                                    DevStatus* st, u32* over) {
   __shared__ HotSums<kGbHotLog2> hot;
   hot.clear();
   __syncthreads();
-  const u64 mask = (1ULL << log2cap) - 1;
+  const u64 mask = (1ULL << t.log2cap) - 1;
   const u64 limit = over ? min(mask, kGbMaxProbes - 1) : mask;
-  const bool use_hot = log2cap < 32;
+  const bool use_hot = t.log2cap < 32;
   gb_each_run<TK, TV, VEC>(key, val, n, st, [&](i64 k, i64 acc) {
-    u64 s = slot_hash(k) & mask;
-    u64 probes = 0;
-    for (; probes <= limit; ++probes) {
-      i64 cur = slots[2 * s];  // a stale free slot is seen by the CAS
-      if (cur == kEmpty) cur = (i64)atomicCAS((u64*)&slots[2 * s], (u64)kEmpty, (u64)k);
-      if (cur == kEmpty || cur == k) break;
-      if (over && (probes & 7) == 7 && *(volatile u32*)over) return;
-      s = (s + 1) & mask;
-    }
-    if (probes > limit) {
-      if (over) *(volatile u32*)over = 1;
-      else latch(st, PQ_ERR_CAPACITY, -1);
-      return;
-    }
-    if (use_hot && hot.add((u32)s, acc, hot.owner((u32)s))) return;
-    atomicAdd((u64*)&slots[2 * s + 1], (u64)acc);
+    const u64 s = gb_slot<STRIDE>(t, k, mask, limit, over, st);
+    if (s == ~0ULL || (use_hot && hot.add((u32)s, acc, hot.owner((u32)s)))) return;
+    atomicAdd((u64*)&t.sums[STRIDE * s], (u64)acc);
   });
-  __syncthreads();
-  for (int i = threadIdx.x; i < hot.kN; i += blockDim.x)
-    if (hot.key[i] != kHotFree)
-      atomicAdd((u64*)&slots[2 * (u64)hot.key[i] + 1], (u64)hot.hi[i] << 32 | hot.lo[i]);
+  gb_flush<STRIDE>(hot, t);
 }
 
-__global__ void k_gb_clear(longlong2* __restrict__ p, i64 n) {
+// kEmpty in every key, 0 in every sum (sums = keys + 1, or keys + the slots).
+__global__ void k_gb_clear(longlong2* __restrict__ p, i64 n, int pairs) {
   const i64 stride = (i64)gridDim.x * blockDim.x;
   for (i64 i = (i64)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride)
-    p[i] = make_longlong2(kEmpty, 0);
+    p[i] = pairs || 2 * i < n ? make_longlong2(kEmpty, pairs ? 0 : kEmpty) : make_longlong2(0, 0);
 }
+
 
 // The slot array's kernels take `if_over`: with it they run only if the flag
 // is set (the hash table before them did not hold the groups).
@@ -1717,31 +1825,42 @@ __global__ void k_gb_zero_if(longlong2* __restrict__ p, i64 n, const u32* if_ove
 // Dense keys (a key range of at most 4 rows per key): the group of key k is
 // slot k - min, its sum in a zeroed array and its existence in a bitmap, so
 // a run costs one reduction and one bit, at addresses that follow the key
-// order.
-template <typename TK, typename TV, bool VEC>
+// order.  HOT: with the table of frequent groups, where the sample met a
+// frequent key (without one it costs up to a tenth).  A small bitmap's words
+// are looked at before a bit is set: 1000 groups keep theirs in 32 words, on
+// which 8M rows waited for each other 1.6 ms.
+constexpr u64 kGbAskSpan = 1 << 16;
+template <typename TK, typename TV, bool VEC, bool HOT>
 __global__ void __launch_bounds__(256) k_gb_dense(const TK* __restrict__ key,
                                                   const TV* __restrict__ val, i64 n, u64 umin,
                                                   u64 span, i64* __restrict__ sums,
                                                   u32* __restrict__ bm, DevStatus* st,
                                                   const u32* if_over) {
   if (if_over && !*if_over) return;
-  __shared__ HotSums<kGbHotLog2> hot;
-  hot.clear();
-  __syncthreads();
-  const bool use_hot = span < kHotFree;
+  const bool ask = span <= kGbAskSpan;
   auto add = [&](u64 idx, i64 acc) {
     atomicAdd(reinterpret_cast<unsigned long long*>(sums + idx), (unsigned long long)acc);
-    atomicOr(bm + (idx >> 5), 1u << (idx & 31));
+    const u32 bit = 1u << (idx & 31);
+    if (!ask || !(__ldcg(bm + (idx >> 5)) & bit)) atomicOr(bm + (idx >> 5), bit);
   };
-  gb_each_run<TK, TV, VEC>(key, val, n, st, [&](i64 k, i64 acc) {
-    const u64 idx = gb_ukey(k) - umin;
-    if (use_hot && hot.add((u32)idx, acc, hot.owner((u32)idx))) return;
-    add(idx, acc);
-  });
-  __syncthreads();
-  for (int i = threadIdx.x; i < hot.kN; i += blockDim.x)
-    if (hot.key[i] != kHotFree)
-      add(hot.key[i], (i64)((u64)hot.hi[i] << 32 | hot.lo[i]));
+  if constexpr (HOT) {
+    __shared__ HotSums<kGbHotLog2> hot;
+    hot.clear();
+    __syncthreads();
+    const bool use_hot = span < kHotFree;
+    gb_each_run<TK, TV, VEC>(key, val, n, st, [&](i64 k, i64 acc) {
+      const u64 idx = gb_ukey(k) - umin;
+      if (use_hot && hot.add((u32)idx, acc, hot.owner((u32)idx))) return;
+      add(idx, acc);
+    });
+    __syncthreads();
+    for (int i = threadIdx.x; i < hot.kN; i += blockDim.x)
+      if (hot.key[i] != kHotFree)
+        add(hot.key[i], (i64)((u64)hot.hi[i] << 32 | hot.lo[i]));
+  } else {
+    gb_each_run<TK, TV, VEC>(key, val, n, st,
+                             [&](i64 k, i64 acc) { add(gb_ukey(k) - umin, acc); });
+  }
 }
 
 // Positions for a block's outputs, cnt per thread: one atomic on the
@@ -1794,20 +1913,28 @@ __global__ void __launch_bounds__(256) k_gb_dense_emit(const u32* __restrict__ b
 // The groups of the hash table: a thread takes kGbEmitPer consecutive slots
 // and writes their groups at consecutive positions reserved per block step.
 constexpr int kGbEmitPer = 8;
-__global__ void __launch_bounds__(256) k_gb_emit(const longlong2* __restrict__ tab, i64 slots,
-                                                 i64* __restrict__ out_keys,
+template <int STRIDE>
+__global__ void __launch_bounds__(256) k_gb_emit(GbTable t, i64* __restrict__ out_keys,
                                                  i64* __restrict__ out_sums, i64 cap,
                                                  u64* d_ngroups, const u32* over) {
   if (over && *over) return;
-  const i64 step = (i64)gridDim.x * blockDim.x * kGbEmitPer;
+  const i64 slots = 1LL << t.log2cap, step = (i64)gridDim.x * blockDim.x * kGbEmitPer;
   for (i64 b0 = (i64)blockIdx.x * blockDim.x * kGbEmitPer; b0 < slots; b0 += step) {  // block-uniform
     const i64 b = b0 + (i64)threadIdx.x * kGbEmitPer;
     longlong2 e[kGbEmitPer];  // the slots are a power of two, 64 at least
     u32 m = 0;
 #pragma unroll
-    for (int j = 0; j < kGbEmitPer; ++j) e[j] = __ldcs(tab + min(b + j, slots - 1));
+    for (int j = 0; j < kGbEmitPer; ++j) {
+      const i64 at = min(b + j, slots - 1);
+      if (STRIDE == 2) e[j] = __ldcs(reinterpret_cast<const longlong2*>(t.keys) + at);
+      else e[j].x = __ldcs(t.keys + at);
+    }
 #pragma unroll
     for (int j = 0; j < kGbEmitPer; ++j) m |= (u32)(b + j < slots && e[j].x != kEmpty) << j;
+    if (STRIDE == 1)
+#pragma unroll
+      for (int j = 0; j < kGbEmitPer; ++j)
+        if ((m >> j) & 1u) e[j].y = __ldcs(t.sums + b + j);
     u64 pos = block_reserve(d_ngroups, (u32)__popc(m));
 #pragma unroll
     for (int j = 0; j < kGbEmitPer; ++j)
@@ -2498,32 +2625,44 @@ pq_status pq_groupby_sum(pq_ctx* ctx, pq_col key, pq_col val, int64_t* out_keys,
   const i64 slots = (i64)1 << log2cap;
   pqh::Scratch tscr(ctx, s);
   auto table = [&]() { return (i64*)tscr.get((size_t)slots * 16); };
-  // Clear and fill the hash table.  At least 128 rows per warp; few rows are
-  // not worth a block each.
+  const bool pairs = (size_t)slots * 16 > kGbPairBytes;
+  auto layout = [&](i64* tab) {
+    return GbTable{tab, tab + (pairs ? 1 : slots), log2cap};
+  };
+  // Clear and fill the hash table; runs: at least 128 rows per warp.
   const int grid = (int)std::min<i64>((key.n + 1023) / 1024, (i64)ctx->num_sms * 6);
-  auto insert = [&](i64* tab, u32* over) -> pq_status {
+  const int grid1 = (int)std::min<i64>((key.n + 255) / 256, (i64)ctx->num_sms * 8);
+  auto insert = [&](i64* tab, bool hot, u32* over) -> pq_status {
     k_gb_clear<<<(int)std::min<i64>((slots + 255) / 256, (i64)ctx->num_sms * 8), 256, 0, s>>>(
-        (longlong2*)tab, slots);
+        (longlong2*)tab, slots, pairs);
     PQ_LAUNCHED(ctx);
     PQ_DISPATCH_T(key.type, TK, {
       PQ_DISPATCH_T(val.type, TV, {
-        auto ins = [&](auto k) {
-          k<<<grid, 256, 0, s>>>((const TK*)key.data, (const TV*)val.data, key.n, tab, log2cap,
-                                 ctx->d_status, over);
+        auto ins = [&](auto k, int g) {
+          k<<<g, 256, 0, s>>>((const TK*)key.data, (const TV*)val.data, key.n, layout(tab),
+                              ctx->d_status, over);
         };
-        vec ? ins(k_gb_insert<TK, TV, true>) : ins(k_gb_insert<TK, TV, false>);
+        if (!hot)
+          pairs ? ins(k_gb_rows<TK, TV, 2>, grid1) : ins(k_gb_rows<TK, TV, 1>, grid1);
+        else if (vec)
+          pairs ? ins(k_gb_insert<TK, TV, true, 2>, grid) : ins(k_gb_insert<TK, TV, true, 1>, grid);
+        else
+          pairs ? ins(k_gb_insert<TK, TV, false, 2>, grid) : ins(k_gb_insert<TK, TV, false, 1>, grid);
       });
     });
     PQ_LAUNCHED(ctx);
     return PQ_OK;
   };
-  auto emit = [&](const i64* tab, const u32* over) -> pq_status {
+  auto emit = [&](i64* tab, const u32* over) -> pq_status {
     const int g = (int)std::min<i64>((slots + 2047) / 2048, (i64)ctx->num_sms * 8);
-    k_gb_emit<<<g, 256, 0, s>>>((const longlong2*)tab, slots, (i64*)out_keys, (i64*)out_sums, cap,
-                                (u64*)d_ngroups, over);
+    auto em = [&](auto k) {
+      k<<<g, 256, 0, s>>>(layout(tab), (i64*)out_keys, (i64*)out_sums, cap, (u64*)d_ngroups, over);
+    };
+    pairs ? em(k_gb_emit<2>) : em(k_gb_emit<1>);
     PQ_LAUNCHED(ctx);
     return PQ_OK;
   };
+  bool hot = false;  // a sample met a frequent key
   // Large inputs outside stream capture: one read of the keys and one small
   // read-back tell whether they come in order (groups are then their runs),
   // and their range; dense keys take the slot array.
@@ -2541,8 +2680,8 @@ pq_status pq_groupby_sum(pq_ctx* ctx, pq_col key, pq_col val, int64_t* out_keys,
       PQ_CUDA(ctx, cudaMemsetAsync(sum, 0, sizeof(GbSummary), s));
       PQ_CUDA(ctx, cudaMemsetAsync(&sum->umin, 0xFF, 8, s));
       PQ_DISPATCH_T(key.type, TK, {
-        if (vec) k_gb_scan<TK, true><<<g, 256, 0, s>>>((const TK*)key.data, key.n, winfo, sum);
-        else k_gb_scan<TK, false><<<g, 256, 0, s>>>((const TK*)key.data, key.n, winfo, sum);
+        if (vec) k_gb_scan<TK, true><<<g + 1, 256, 0, s>>>((const TK*)key.data, key.n, winfo, sum);
+        else k_gb_scan<TK, false><<<g + 1, 256, 0, s>>>((const TK*)key.data, key.n, winfo, sum);
       });
       PQ_LAUNCHED(ctx);
       k_gb_bounds<<<1, 1024, 0, s>>>(winfo, nw, base, sum);
@@ -2552,6 +2691,7 @@ pq_status pq_groupby_sum(pq_ctx* ctx, pq_col key, pq_col val, int64_t* out_keys,
       PQ_CUDA(ctx, cudaStreamSynchronize(s));
       GbSummary m;
       memcpy(&m, hp.p, sizeof m);
+      hot = m.top >= kGbTopHot;
       // In order, or in order but for one descent with few runs after it (a
       // late part appended to an ordered table); the reserved key (ukey 0)
       // goes to the tables, which report it.
@@ -2597,18 +2737,21 @@ pq_status pq_groupby_sum(pq_ctx* ctx, pq_col key, pq_col val, int64_t* out_keys,
         const size_t bb = (size_t)(((span + 31) / 32 * 4 + 255) / 256 * 256);
         char* blk = (char*)scr.get(sb + bb);
         if (blk) {
-          // Rows in no order touch their groups at random: what counts is how
-          // much memory the groups take (30M Zipf rows, 7.5M groups in a range
-          // of 30M: slot array of 240 MB 0.94 ms, hash table of 134 MB 0.45
-          // ms).  Rows in runs follow the slot array's order.  The hash table
-          // holds `cap` groups; the slot array takes over, decided on the
-          // device, when there are more, as every group is counted.
-          i64* const tab = m.runs > key.n / 2 && span > (u64)slots ? table() : nullptr;
+          // Rows in no order with frequent keys: what counts is how much memory
+          // the other groups take (30M Zipf rows, 7.5M groups in a range of 30M:
+          // slot array of 240 MB 0.94 ms, hash table of 134 MB 0.45 ms).  Without
+          // frequent keys the slot array's reductions, which nobody waits for,
+          // are ahead of the look-ups whatever their memory (40M rows, 400000
+          // groups in a range of 26M: 0.62 ms, hash table of 16 MB 0.96 ms), and
+          // rows in runs follow its order.  The hash table holds `cap` groups; the
+          // slot array takes over, decided on the device, when there are more, as
+          // every group is counted.
+          i64* const tab = hot && m.runs > key.n / 2 && span > (u64)slots ? table() : nullptr;
           u32* const over = tab ? &sum->over : nullptr;
           i64* sums = (i64*)blk;
           u32* bm = (u32*)(blk + sb);
           if (tab) {
-            const pq_status st = insert(tab, over);
+            const pq_status st = insert(tab, hot, over);
             if (st != PQ_OK) return st;
             k_gb_zero_if<<<ctx->num_sms * 8, 256, 0, s>>>((longlong2*)blk, (i64)((sb + bb) / 16),
                                                           over);
@@ -2618,11 +2761,14 @@ pq_status pq_groupby_sum(pq_ctx* ctx, pq_col key, pq_col val, int64_t* out_keys,
           }
           PQ_DISPATCH_T(key.type, TK, {
             PQ_DISPATCH_T(val.type, TV, {
+              const int gd = hot ? grid : (int)std::min<i64>((key.n + 1023) / 1024,
+                                                             (i64)ctx->num_sms * 8);
               auto dense = [&](auto k) {
-                k<<<grid, 256, 0, s>>>((const TK*)key.data, (const TV*)val.data, key.n, m.umin,
+                k<<<gd, 256, 0, s>>>((const TK*)key.data, (const TV*)val.data, key.n, m.umin,
                                        span, sums, bm, ctx->d_status, over);
               };
-              vec ? dense(k_gb_dense<TK, TV, true>) : dense(k_gb_dense<TK, TV, false>);
+              if (hot) vec ? dense(k_gb_dense<TK, TV, true, true>) : dense(k_gb_dense<TK, TV, false, true>);
+              else vec ? dense(k_gb_dense<TK, TV, true, false>) : dense(k_gb_dense<TK, TV, false, false>);
             });
           });
           PQ_LAUNCHED(ctx);
@@ -2645,7 +2791,7 @@ pq_status pq_groupby_sum(pq_ctx* ctx, pq_col key, pq_col val, int64_t* out_keys,
   i64* const tab = table();
   if (!tab) return pqh::fail(ctx, PQ_ERR_BUDGET, "pq_groupby_sum: table of %lld slots",
                              (long long)slots);
-  pq_status st = insert(tab, nullptr);
+  pq_status st = insert(tab, hot, nullptr);
   if (st == PQ_OK) st = emit(tab, nullptr);
   if (st != PQ_OK) return st;
   k_check_cap<<<1, 1, 0, s>>>((const i64*)d_ngroups, cap, ctx->d_status);
