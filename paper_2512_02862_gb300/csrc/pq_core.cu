@@ -91,6 +91,27 @@ void* Arena::alloc(size_t bytes, size_t align) {
   }
 }
 
+void* Arena::alloc_top(size_t bytes) {
+  std::lock_guard<std::mutex> g(mu_);
+  bytes = round_up(bytes ? bytes : 1, 256);
+  reclaim(false);
+  if (free_.empty()) return nullptr;
+  const auto it = std::prev(free_.end());
+  const size_t off = it->first, end = off + it->second;
+  // The highest 256-byte boundary that leaves room.
+  const size_t at = bytes <= end ? (size_t)((uintptr_t)(base_ + end - bytes) & ~(uintptr_t)255) -
+                                       (size_t)(uintptr_t)base_
+                                 : 0;
+  if (bytes > end || at < off || at > end) return nullptr;
+  free_.erase(it);
+  if (at > off) free_[off] = at - off;
+  if (at + bytes < end) free_[at + bytes] = end - (at + bytes);
+  live_[at] = bytes;
+  in_use_ += bytes;
+  high_ = std::max(high_, in_use_);
+  return base_ + at;
+}
+
 size_t Arena::largest_free() {
   std::lock_guard<std::mutex> g(mu_);
   reclaim(false);

@@ -2,6 +2,7 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <atomic>
 #include <condition_variable>
 #include <cstdint>
@@ -37,6 +38,8 @@ class Arena {
   size_t in_use() const { return in_use_; }
   size_t high_water() const { return high_; }
   size_t capacity() const { return cap_; }
+  // From the end of the highest free piece; nullptr when it is too small.
+  void* alloc_top(size_t bytes);
   size_t largest_free();
 
  private:
@@ -320,6 +323,18 @@ struct Scratch {
     void* p = ctx->arena.alloc(bytes ? bytes : 256);
     if (p) blocks.push_back(p);
     return p;
+  }
+  // From the arena's end, so that giving it back (drop) joins the room that
+  // blocks taken meanwhile have left.
+  void* get_top(size_t bytes) {
+    void* p = ctx->arena.alloc_top(bytes);
+    if (p) blocks.push_back(p);
+    return p;
+  }
+  // Gives one block back at once: nothing on the device uses it any more.
+  void drop(void* p) {
+    blocks.erase(std::remove(blocks.begin(), blocks.end(), p), blocks.end());
+    ctx->arena.release_now(p);
   }
   ~Scratch() {
     for (void* p : blocks) ctx->arena.release(p, s);

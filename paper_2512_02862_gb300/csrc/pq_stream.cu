@@ -199,7 +199,7 @@ class Stager {
 class BlockTables {
  public:
   // rows[t]: the rows of table t that are streamed (from tabs[t].row0); 0: none.
-  BlockTables(Scratch& scr, const TableIn* tabs, const i64* rows) : tabs_(tabs) {
+  BlockTables(Scratch& scr, const TableIn* tabs, const i64* rows) : scr_(scr), tabs_(tabs) {
     size_t bytes = 0;
     for (int t = 0; t < 3; ++t) {
       if (!tabs[t].packed || rows[t] <= 0) continue;
@@ -208,7 +208,8 @@ class BlockTables {
       bytes += al((size_t)nb_[t] * sizeof(PackBlock)) * tabs[t].ncols;
     }
     // Not from an arena that is nearly used up: the tables sized later need it.
-    char* p = bytes && bytes <= scr.ctx->arena.largest_free() / 64 ? (char*)scr.get(bytes) : nullptr;
+    char* p = bytes && bytes <= scr.ctx->arena.largest_free() / 64 ? (char*)scr.get_top(bytes) : nullptr;
+    mem_ = p;
     for (int t = 0; p && t < 3; ++t) {
       if (!nb_[t]) continue;
       if (cudaEventCreateWithFlags(&ready_[t], cudaEventDisableTiming) != cudaSuccess) {
@@ -228,6 +229,18 @@ class BlockTables {
     }
   }
   BlockTables(const BlockTables&) = delete;
+  // Scratch of a size known only after a scan.  Where the arena has no room for
+  // it the block tables make some: the chunks that are on their way are waited
+  // for, and the others bring their entries along.
+  char* get(size_t bytes) {
+    char* p = (char*)scr_.get(bytes);
+    if (p || !mem_) return p;
+    for (cudaStream_t cs : scr_.ctx->copy_streams) cudaStreamSynchronize(cs);
+    for (char*& at : at_) at = nullptr;
+    scr_.drop(mem_);
+    mem_ = nullptr;
+    return (char*)scr_.get(bytes);
+  }
   // Before a chunk of table t goes out on stream cs: the first one copies the
   // table's entries (their bytes are added to *total), later ones wait for them.
   cudaError_t use(int t, cudaStream_t cs, size_t* total) {
@@ -252,7 +265,9 @@ class BlockTables {
   }
 
  private:
+  Scratch& scr_;
   const TableIn* tabs_;
+  char* mem_ = nullptr;
   char* at_[3] = {};
   i64 b0_[3] = {}, nb_[3] = {};
   cudaEvent_t ready_[3] = {};
@@ -553,7 +568,7 @@ pq_status run_plan_streaming(pq_ctx* ctx, const pq_plan* plan, pq_result* result
     }
     const int e = cap_log2(count, d.lf1024);
     if (t == 0) {
-      char* blk = (char*)scr.get(dset_block_bytes(e));
+      char* blk = btabs.get(dset_block_bytes(e));
       if (!blk) return fail(ctx, PQ_ERR_BUDGET, "streaming plan: D-set of 2^%d slots", e);
       dset_block_assign(blk, e, d);
       PQ_CUDA(ctx, upload_desc(0, r.resident[1] ? (r.n_m + d.m_tile - 1) / d.m_tile : 0,
@@ -568,8 +583,7 @@ pq_status run_plan_streaming(pq_ctx* ctx, const pq_plan* plan, pq_result* result
       }
     } else {
       const i64 parts = topk_parts(e), cap = topk_cand_cap(e, d.k);
-      char* blk = (char*)scr.get(mtable_bytes(e) + al(parts * 4) +
-                                 al(cap * 8) * 2);
+      char* blk = btabs.get(mtable_bytes(e) + al(parts * 4) + al(cap * 8) * 2);
       if (!blk) return fail(ctx, PQ_ERR_BUDGET, "streaming plan: M table of 2^%d slots", e);
       char* p = mtable_assign(blk, e, d);
       d.tk_c = (int*)p;
@@ -920,15 +934,14 @@ pq_status run_batch_streaming(pq_ctx* ctx, const pq_plan* plans, int n, pq_resul
       const i64 count = (i64)(t == 0 ? hctr[i].dcount : hctr[i].mcount);
       const int e = cap_log2(count, d.lf1024);
       if (t == 0) {
-        char* blk = (char*)scr.get(dset_block_bytes(e));
+        char* blk = btabs.get(dset_block_bytes(e));
         if (!blk) return fail(ctx, PQ_ERR_BUDGET, "streaming batch: D-set of 2^%d slots", e);
         dset_block_assign(blk, e, d);
         // The D scan's last block wrote the header into the placeholder.
         PQ_CUDA(ctx, cudaMemcpyAsync(d.dset_log2, dset_ph[i], 24, cudaMemcpyDeviceToDevice, s));
       } else {
         const i64 parts = topk_parts(e), cap = topk_cand_cap(e, d.k);
-        char* blk = (char*)scr.get(mtable_bytes(e) + al(parts * 4) +
-                                   al(cap * 8) * 2);
+        char* blk = btabs.get(mtable_bytes(e) + al(parts * 4) + al(cap * 8) * 2);
         if (!blk) return fail(ctx, PQ_ERR_BUDGET, "streaming batch: M table of 2^%d slots", e);
         char* p = mtable_assign(blk, e, d);
         d.tk_c = (int*)p;
