@@ -1057,12 +1057,12 @@ __device__ __forceinline__ u64 ht_first(const HtMeta& m, i64 k, u64 mask) {
   const u64 d = ((u64)k ^ 0x8000000000000000ULL) - m.umin;
   return d <= m.range ? __umul64hi(d, m.scale) : slot_hash(k) & mask;
 }
-// Slot i of the path from slot i - 1.
-__device__ __forceinline__ u64 ht_next(u64 s, i64 k, u64 i, u64 mask) {
-  const u64 pos = (s + 1) & 7;
-  if (i & 7) return (s & ~7ULL) | pos;
+// Slot i of the path that starts at slot s.
+__device__ __forceinline__ u64 ht_line_slot(u64 s, u64 i) { return (s & ~7ULL) | ((s + i) & 7); }
+__device__ __forceinline__ u64 ht_slot(u64 s, i64 k, u64 i, u64 mask) {
+  if (i < 8) return ht_line_slot(s, i);
   const u64 step = __umul64hi(0x9E3779B97F4A7C15ULL, (mask + 1) >> 3) | 1;
-  return (((slot_hash(k) >> 20) + (i - 8) * step) & mask & ~7ULL) | pos;
+  return (((slot_hash(k) >> 20) + ((i & ~7ULL) - 8) * step) & mask & ~7ULL) | ((s + i) & 7);
 }
 
 // 512 build keys spread over the input (the first and the last among them):
@@ -1197,14 +1197,14 @@ __global__ void __launch_bounds__(256) k_ht_build_spread(const TK* __restrict__ 
 #pragma unroll
     for (int h = 0; h < kBldKeys; ++h) {
       if (k[h] == kEmpty) continue;
-      u64 probes = 0;
+      u64 probes = 0, at = s[h];
       while (old[h] != kEmpty) {
         if (old[h] == k[h]) meta->dup = 1;
         if (++probes > mask + 8) break;
-        s[h] = ht_next(s[h], k[h], probes, mask);
-        old[h] = (i64)atomicCAS((u64*)&slots[2 * s[h]], (u64)kEmpty, (u64)k[h]);
+        at = ht_slot(s[h], k[h], probes, mask);
+        old[h] = (i64)atomicCAS((u64*)&slots[2 * at], (u64)kEmpty, (u64)k[h]);
       }
-      if (old[h] == kEmpty) slots[2 * s[h] + 1] = v[h];
+      if (old[h] == kEmpty) slots[2 * at + 1] = v[h];
       else latch(st, PQ_ERR_CAPACITY, i0 + h * stride);
     }
   }
@@ -1218,10 +1218,11 @@ __global__ void __launch_bounds__(256) k_ht_build_spread(const TK* __restrict__ 
 // reservation per pair-producing round would make that counter the bound
 // (millions of atomics on one address).  Blocks of 8 warps, one resident
 // wave, five of them per SM (48 registers).  60M rows in key order against
-// 15M build keys: 1.01 ms hashed, 0.55 ms with lines in key order (four rows
-// per lane at 64 registers, which the hashed loop cannot spare: 0.51 ms).  The hashed loop is a function of its own:
-// inlined with the other one it was 9 % slower, and as two kernels of which one
-// returns at once a probe took 6 us more.
+// 15M build keys: 1.00 ms hashed, 0.46 ms with lines in key order, whose first 8
+// slots are a loop without the hash of the rest of the path (with it 0.55 ms;
+// four rows per lane at 64 registers 0.48 ms).  The hashed loop is a function of
+// its own: inlined with the other one it was 9 % slower, and as two kernels of
+// which one returns at once a probe took 6 us more.
 constexpr int kPrbBuf = 256, kPrbBlocks = 5;
 struct PrbStage {
   i64 row[8][kPrbBuf], val[8][kPrbBuf];
@@ -1265,45 +1266,45 @@ __device__ __forceinline__ void ht_probe(const TK* __restrict__ pkey, i64 n,
       if (k[h] == kEmpty) active[h] = false;
       s[h] = SPREAD ? ht_first(m, k[h], mask) : slot_hash(k[h]) & mask;
     }
-    // Slot j of both rows; fresh(h, j): the slot is met for the first time,
-    // next(h, j): the one after it.
-    auto step = [&](u64 j, auto fresh, auto next) {
+    // The two rows' slots at(h); met(h): the slot was met before on the path.
+    auto step = [&](auto at, auto met) {
       longlong2 kv[2];  // {key, value} of each row's current slot
 #pragma unroll
-      for (int h = 0; h < 2; ++h) kv[h] = active[h] ? __ldg(slots + s[h]) : make_longlong2(kEmpty, 0);
+      for (int h = 0; h < 2; ++h)
+        kv[h] = active[h] ? __ldg(slots + at(h)) : make_longlong2(kEmpty, 0);
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         bool emit = false;
         if (active[h]) {
           if (kv[h].x == kEmpty) {
             active[h] = false;
-          } else {
-            if (kv[h].x == k[h] && fresh(h, j)) {
-              emit = true;
-              if (!dup) active[h] = false;
-            }
-            s[h] = next(h, j);
+          } else if (kv[h].x == k[h] && !met(h)) {
+            emit = true;
+            if (!dup) active[h] = false;
           }
         }
         const u32 em = __ballot_sync(kFull, emit);
         if (emit) {
-          const u32 at = nb + __popc(em & lanemask_lt());
-          br[at] = i[h], bv[at] = kv[h].y;
+          const u32 to = nb + __popc(em & lanemask_lt());
+          br[to] = i[h], bv[to] = kv[h].y;
         }
         nb += __popc(em);
       }
       if (nb > kPrbBuf - 64) flush();  // room for a full round stays
     };
     if constexpr (SPREAD) {
-      for (u64 j = 0; j <= mask + 8 && __any_sync(kFull, active[0] || active[1]); ++j)
-        step(j,
-             [&](int h, u64 jj) {  // (the path may come by the first line again)
-               return jj < 8 || ((s[h] ^ ht_first(m, k[h], mask)) & ~7ULL);
-             },
-             [&](int h, u64 jj) { return ht_next(s[h], k[h], jj + 1, mask); });
+      for (u32 j = 0; j < 8 && __any_sync(kFull, active[0] || active[1]); ++j)
+        step([&](int h) { return ht_line_slot(s[h], j); }, [](int) { return false; });
+      // Past a full line (the path may come by it again).
+      for (u64 j = 8; j <= mask + 8 && __any_sync(kFull, active[0] || active[1]); ++j)
+        step([&](int h) { return ht_slot(s[h], k[h], j, mask); },
+             [&](int h) { return !((ht_slot(s[h], k[h], j, mask) ^ s[h]) & ~7ULL); });
     } else {
-      while (__any_sync(kFull, active[0] || active[1]))  // a slot is always free
-        step(0, [](int, u64) { return true; }, [&](int h, u64) { return (s[h] + 1) & mask; });
+      while (__any_sync(kFull, active[0] || active[1])) {  // a slot is always free
+        step([&](int h) { return s[h]; }, [](int) { return false; });
+#pragma unroll
+        for (int h = 0; h < 2; ++h) s[h] = (s[h] + 1) & mask;
+      }
     }
   }
   if (nb) flush();

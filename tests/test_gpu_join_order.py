@@ -120,3 +120,32 @@ def test_even_keys_with_strays(ctx, stream):
     build[at[100:]] = 2**62 + np.arange(100)
     probe = np.concatenate([build, build + 1, [-2**63 + 1, 2**63 - 1, 2**62 + 50]])
     check_join(ctx, stream, build, np.arange(n), probe)
+
+
+@pytest.mark.parametrize("kind", ["even", "shuffled", "repeated"])
+def test_tens_of_millions_of_probes(ctx, stream, kind):
+    """Many rounds per warp: every match once, compared on the device."""
+    n, m = 1_000_000, 2**25 + 77
+    g = torch.Generator(device="cuda")
+    g.manual_seed(5)
+    build = torch.arange(n, device="cuda") * 4 + torch.randint(0, 4, (n,), generator=g, device="cuda")
+    at = torch.randint(0, n, (m,), generator=g, device="cuda")
+    probe = build[at]
+    probe[::5] = -7
+    if kind == "repeated":  # each of 1000 keys twice
+        build[n - 1000:] = build[:1000]
+        probe = torch.where(at >= n - 1000, torch.full_like(probe, -7), probe)
+    order = torch.randperm(n, generator=g, device="cuda") if kind != "even" else torch.arange(n, device="cuda")
+    copies = torch.where(probe == -7, 0, torch.where(at < 1000, 2 if kind == "repeated" else 1, 1))
+    pairs = int(copies.sum())
+    torch.cuda.synchronize()
+    with torch.cuda.stream(stream):
+        ht = pq.pq_join_build(ctx, build[order].contiguous(), order, stream=stream)
+        r, w, cnt = pq.pq_join_probe(ctx, ht, probe, pairs, stream=stream)
+        ht.free(stream)
+        ctx.sync(stream)
+    assert int(cnt.item()) == pairs
+    assert bool((torch.bincount(r, minlength=m) == copies).all())
+    assert bool((build[w] == probe[r]).all())
+    # Pairs are distinct: a row's two matches are different build rows.
+    assert torch.unique(r * n + w).numel() == pairs
