@@ -2243,9 +2243,10 @@ pq_status pq_filter(pq_ctx* ctx, pq_col col, int op, int64_t c, const int64_t* s
   // At least two warp tiles per warp, at most one wave of blocks.
   const int g = (int)std::max<i64>(1, std::min<i64>((wtiles + 15) / 16,
                                                        (i64)ctx->num_sms * filter_blocks(sel || col.type == PQ_INT64)));
-  // Scratch of a capture is kept for the graph's replays: only the counts.
+  // Scratch of a capture is kept for the graph's replays: only the counts (the
+  // bits of 2^18 rows take as much; small calls do not ask, it costs 1 us).
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  cudaStreamIsCapturing(s, &cap);
+  if (n_cap > 1 << 18) cudaStreamIsCapturing(s, &cap);
   const bool keep = cap == cudaStreamCaptureStatusNone;
   const size_t bits_b = keep ? (size_t)wtiles * 64 : 0, cnt_b = (size_t)g * 9 * 4;
   if (char* w = in_place ? nullptr : (char*)scr.get(bits_b + cnt_b)) {
@@ -2416,11 +2417,12 @@ pq_status part_pass(pq_ctx* ctx, pq_col key, const pq_col* payload, int npay, Di
 // per bucket and sub-tile, where one pass by 1024 buckets writes runs of two
 // to four (partly written sectors, and 8 x 1024 counters a sub-tile that leave
 // room for one block per SM), and above that 8192-row tiles are scattered row
-// by row.  It moves the rows twice and takes nine more launches, so it pays
-// from some size on.  20M rows of 21 bytes by 1024: 0.67 -> 0.46 ms, 60M of
-// 16 bytes 1.10 -> 1.02 ms (20M of them 0.41 either way; by 512 buckets one
-// pass is faster, 0.98 against 0.99 ms); 20M rows of 16 bytes by 2048 0.65 -> 0.42 ms, by
-// 4096 1.33 -> 0.43 ms; 4M of them by 2048 0.18 -> 0.17 ms, by 4096 0.31 -> 0.17.
+// by row.  It moves the rows twice and takes six more launches and clears, so it
+// pays from some size on.  Uniform keys, 20M rows of 21 bytes by 1024: 0.94 ->
+// 0.46 ms (clustered keys 0.67 -> 0.44), 60M of 16 bytes 1.20 -> 0.99 ms (20M of
+// them 0.40 either way; by 512 buckets one pass is faster, 0.97 against 0.99 ms);
+// 20M rows of 16 bytes by 2048 0.94 -> 0.40 ms, by 4096 1.44 -> 0.41 ms; 4M of
+// them by 2048 0.22 -> 0.15 ms, by 4096 0.34 -> 0.16.
 bool part_two_passes(int log2P, i64 n, const pq_col& key, const pq_col* payload, int npay) {
   i64 row = (i64)pqh::dtype_size(key.type);
   for (int j = 0; j < npay; ++j) row += (i64)pqh::dtype_size(payload[j].type);
@@ -2821,11 +2823,12 @@ pq_status pq_topk(pq_ctx* ctx, const int64_t* keys, const int64_t* sums, int64_t
 }  // extern "C"
 
 // ===================================================== allocation-free filter ====
-// pq_filter needs scratch for its single-pass tile prefixes, normally carved
-// from the context's arena.  Some callers cannot allocate device memory at all
-// (for example code that runs while a CUDA graph is being captured, or inside
-// a runtime that owns every allocation and forbids others), and they may not
-// have a context either.  For them the same kernel runs with its scratch in
+// pq_filter takes its scratch from the context's arena.  Some callers cannot
+// allocate device memory at all (for example code that runs while a CUDA graph
+// is being captured, or inside a runtime that owns every allocation and forbids
+// others), and they may not have a context either.  For them the single-pass
+// kernel with look-back (k_filter, pq_filter's way in place and without scratch
+// for its bits) runs with its tile states in
 // this file-scope device array: a fixed 1 MiB of tile states plus a small
 // header, which every GPU that loads the library keeps until the process
 // exits.  All calls share the array, so calls that overlap on the GPU race;
