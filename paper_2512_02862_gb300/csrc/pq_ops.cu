@@ -2306,6 +2306,7 @@ pq_status pq_filter(pq_ctx* ctx, pq_col col, int op, int64_t c, const int64_t* s
 }  // extern "C"
 
 namespace {
+constexpr int kPartSmem = 200 * 1024;  // most dynamic shared memory of a scatter
 // One stable pass of the partition: rows ordered by digit `dg` of their
 // bucket.  d_offsets: the digits' offsets (or null); tot: null, or counts of
 // whole buckets to be added to (zeroed by the caller).
@@ -2351,8 +2352,8 @@ pq_status part_pass(pq_ctx* ctx, pq_col key, const pq_col* payload, int npay, Di
   size_t smem = layout(sub);
   const int row_bytes = tc.buf_bytes / sub;
   const bool runs = dg.bits >= 9 || (dg.bits == 8 && row_bytes > 4 && row_bytes <= 8);
-  if (!runs || smem > 200 * 1024) smem = layout(sub = kSub);
-  const bool use_tma = aligned && smem <= 200 * 1024;
+  if (!runs || smem > kPartSmem) smem = layout(sub = kSub);
+  const bool use_tma = aligned && smem <= kPartSmem;
   if (!use_tma) sub = kSub, smem = staged_smem(P);
   // Blocks per SM: by shared memory (228 KB, 1 KB and the static part of it
   // taken per block) and, at most, by registers.
@@ -2392,7 +2393,9 @@ pq_status part_pass(pq_ctx* ctx, pq_col key, const pq_col* payload, int npay, Di
         hist, m, gofs, (u64*)(w + 256), (u32*)w, ctx->opt.spin_limit, ctx->d_status);
     PQ_LAUNCHED(ctx);
     auto launch = [&](auto k, auto... args) -> pq_status {
-      PQ_CUDA(ctx, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+      // The same limit on every call, whatever this one needs: another thread may
+      // be between its own setting and its launch.
+      PQ_CUDA(ctx, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kPartSmem));
       k<<<(unsigned)g, 256, smem, s>>>(args...);
       PQ_LAUNCHED(ctx);
       return PQ_OK;

@@ -44,3 +44,35 @@ def test_row_widths(ctx, log2P, kt, pay, off):
     assert np.array_equal(ok.cpu().numpy(), wk)
     for a, b in zip(oc, wc):
         assert np.array_equal(a.cpu().numpy(), b)
+
+
+def test_threads_with_different_shapes():
+    """Two threads, each with a context of its own, partition rows of different
+    widths and bucket counts with the same kernel."""
+    import threading
+
+    n, errors = 300_007, []
+
+    def work(seed, log2P, wide):
+        try:
+            rng = np.random.default_rng(seed)
+            key = rng.integers(-2**40, 2**40, size=n)
+            cols = [rng.integers(0, 100, size=n) for _ in range(3 if wide else 1)]
+            ctx, s = pq.Context(arena_bytes=256 << 20), torch.cuda.Stream()
+            with torch.cuda.stream(s):
+                k, c = torch.from_numpy(key).cuda(), [torch.from_numpy(a).cuda() for a in cols]
+                for _ in range(200):
+                    ok, _, o = pq.pq_partition(ctx, k, c, log2P=log2P, stream=s)
+                ctx.sync(s)
+            wk, _, wo = oracle.partition(key, log2P, cols)
+            assert np.array_equal(o.cpu().numpy(), wo) and np.array_equal(ok.cpu().numpy(), wk)
+            ctx.close()
+        except Exception as e:  # seen by the test's thread
+            errors.append(e)
+
+    threads = [threading.Thread(target=work, args=a) for a in ((1, 7, True), (2, 3, False))]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors
