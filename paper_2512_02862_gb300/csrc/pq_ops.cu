@@ -1401,9 +1401,14 @@ __device__ __forceinline__ void gb_sample(const TK* __restrict__ key, i64 n, GbS
   if (threadIdx.x == 0) sum->top = s_top;
 }
 
-// (The first block samples the keys meanwhile.)
+// The first block samples the keys meanwhile.  Four blocks per SM, of this pass
+// and of the one over the runs, whose shares of the rows are the same: 61
+// registers and one wave.  (Six, which the scan alone would fit, held it to 40
+// registers with 72 bytes of spills and made the runs one wave and a half: 40M
+// ordered rows of 400 groups 198 -> 186 us a call, 8M 78 -> 68.)
+constexpr int kGbScanBlocks = 4;
 template <typename TK, bool VEC>
-__global__ void __launch_bounds__(256, 6) k_gb_scan(const TK* __restrict__ key, i64 n,
+__global__ void __launch_bounds__(256, kGbScanBlocks) k_gb_scan(const TK* __restrict__ key, i64 n,
                                                     GbWarp* __restrict__ wout, GbSummary* sum) {
   if (blockIdx.x == 0) {
     gb_sample(key, n, sum);
@@ -1538,7 +1543,7 @@ __global__ void k_gb_joins(const GbWarp* __restrict__ w, const i64* __restrict__
 // k_gb_scan; the range pass, slot array and its emit took 0.63 ms (and three
 // clears), which unordered rows still take.
 template <typename TK, typename TV, bool VEC>
-__global__ void __launch_bounds__(256, 4) k_gb_runs(const TK* __restrict__ key,
+__global__ void __launch_bounds__(256, kGbScanBlocks) k_gb_runs(const TK* __restrict__ key,
                                                     const TV* __restrict__ val, i64 n,
                                                     const GbWarp* __restrict__ winfo,
                                                     const i64* __restrict__ base, GbOut o) {
@@ -2676,7 +2681,7 @@ pq_status pq_groupby_sum(pq_ctx* ctx, pq_col key, pq_col val, int64_t* out_keys,
   cudaStreamIsCapturing(s, &capst);
   if (capst == cudaStreamCaptureStatusNone && key.n >= (1 << 20)) {
     pqh::Scratch rs(ctx, s);
-    const int g = ctx->num_sms * 6, nw = g * 8;
+    const int g = ctx->num_sms * kGbScanBlocks, nw = g * 8;
     const size_t base_b = 256 + (size_t)(nw + 1) * 8;
     char* w = (char*)rs.get(base_b + (size_t)nw * sizeof(GbWarp));
     if (w) {
