@@ -263,6 +263,7 @@ struct pq_ctx {
   // tuning (kernel launch shapes chosen by pq_autotune or the options)
   int tune_threads = 256;
   int tune_bps = 2;
+  std::atomic<uint32_t> part_ready{0};   // partition kernels whose shared-memory limit is set
   // resident blocks per SM of each plan kernel (filled by plan_kernels_init)
   int plan_occ[28] = {0};
 };

@@ -2397,26 +2397,30 @@ pq_status part_pass(pq_ctx* ctx, pq_col key, const pq_col* payload, int npay, Di
     k_scan_u32<<<(unsigned)std::min<i64>(stiles, (i64)ctx->num_sms * 4), 256, 0, s>>>(
         hist, m, gofs, (u64*)(w + 256), (u32*)w, ctx->opt.spin_limit, ctx->d_status);
     PQ_LAUNCHED(ctx);
-    auto launch = [&](auto k, auto... args) -> pq_status {
-      // The same limit on every call, whatever this one needs: another thread may
-      // be between its own setting and its launch.
-      PQ_CUDA(ctx, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kPartSmem));
+    auto launch = [&](int variant, auto k, auto... args) -> pq_status {
+      // Once per context, and the same limit whatever this call needs: another
+      // thread may be between its own setting and its launch.
+      const uint32_t bit = 1u << ((key.type - 1) * 8 + variant);
+      if (!(ctx->part_ready.load(std::memory_order_acquire) & bit)) {
+        PQ_CUDA(ctx, cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kPartSmem));
+        ctx->part_ready.fetch_or(bit, std::memory_order_release);
+      }
       k<<<(unsigned)g, 256, smem, s>>>(args...);
       PQ_LAUNCHED(ctx);
       return PQ_OK;
     };
     if (!use_tma)
-      return launch(k_part_scatter_blk<T, PART>, (const T*)key.data, n, dg, (const i64*)gofs, pa,
+      return launch(PART ? 1 : 0, k_part_scatter_blk<T, PART>, (const T*)key.data, n, dg, (const i64*)gofs, pa,
                     (T*)out_key, d_offsets);
-    auto scatter = [&](auto k) {
-      return launch(k, n, dg, (const i64*)gofs, tc, d_offsets, (i64)ctx->opt.spin_limit,
+    auto scatter = [&](int variant, auto k) {
+      return launch(variant, k, n, dg, (const i64*)gofs, tc, d_offsets, (i64)ctx->opt.spin_limit,
                     ctx->d_status);
     };
     if constexpr (!PART) {  // a part has 64 digits at most
-      if (sub == 4096) return scatter(k_part_scatter_tma<T, PART, 4096, 3>);
-      if (!bound) return scatter(k_part_scatter_tma<T, PART, kSub, 0>);
+      if (sub == 4096) return scatter(2, k_part_scatter_tma<T, PART, 4096, 3>);
+      if (!bound) return scatter(3, k_part_scatter_tma<T, PART, kSub, 0>);
     }
-    return scatter(k_part_scatter_tma<T, PART, kSub, 3>);
+    return scatter(PART ? 4 : 5, k_part_scatter_tma<T, PART, kSub, 3>);
   });
   return PQ_OK;
 }

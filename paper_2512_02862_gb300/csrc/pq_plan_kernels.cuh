@@ -380,6 +380,9 @@ constexpr int kAT = 1024;
 // whose members are less than one M row in kDirectShare are not looked at
 // further; for the others direct_vote samples F.
 constexpr i64 kDirectShare = 8;
+// Nor are plans whose rows, all joining, would save less than this (0.45M rows):
+// the look costs what the pass could gain (300k rows 99 us either way).
+constexpr i64 kDirectGate = 35000000;
 // The M scan's verdict (Batch::direct_ok plans): a word of the work area, so
 // that the later kernels know it after a single load.
 constexpr int kDirectWord = 32;
@@ -847,7 +850,7 @@ __global__ void __launch_bounds__(256) k_plan_dbuild(Batch b) {
 // that passes the date test and the share that also joins (3 us, for plans that
 // get here).  In bytes of the columns' rate,
 // the pass costs price and discount of every sector with a passing row (four
-// such rows), the sums of all members in the top-k and 5 us of its own; a hit
+// such rows), the sums of all members in the top-k and 3 us of its own; a hit
 // saves 80.  Against the hit list, 40M rows over 10M M rows: 15 % of M and all
 // of F's dates, 344 -> 305 us clustered and 509 -> 393 us Zipf; half of the
 // dates 305 -> 320, a tenth 243 -> 295; 4M rows that all join 197 -> 123, a
@@ -859,7 +862,7 @@ __device__ __noinline__ void direct_vote(const PlanDev* qp, u32* verdict) {
   const i64 members = ld_count(&q.ctr->mcount), n = q.n_f;
   __shared__ u32 s_n[2];
   bool take = members > 0 && members >= q.n_m / kDirectShare &&
-              80 * n > 35000000 + 8 * members && q.rev_max &&
+              80 * n > kDirectGate + 8 * members && q.rev_max &&
               (unsigned __int128)(u64)n * q.rev_max < ((unsigned __int128)1 << 63);
   if (take) {  // block-uniform
     constexpr int kPer = 4;
@@ -892,7 +895,7 @@ __device__ __noinline__ void direct_vote(const PlanDev* qp, u32* verdict) {
     __syncthreads();
     constexpr float kAll = 1.0f / (256 * kPer);
     const float rows = (float)n, f = s_n[0] * kAll, h = s_n[1] * kAll;
-    take = 80.0f * h * rows > 9.0f * rows * fminf(1.0f, 4.0f * f) + 8.0f * members + 3.5e7f;
+    take = 80.0f * h * rows > 9.0f * rows * fminf(1.0f, 4.0f * f) + 8.0f * members + 2e7f;
   }
   if (threadIdx.x == 0) *verdict = take;
 }
