@@ -301,11 +301,10 @@ pq_status pq_join_probe(pq_ctx* ctx, const pq_ht* ht, pq_col probe_key, int64_t*
  * which waits for the stream once: keys in ascending order, but for one late
  * part at most, are grouped by their runs with no table (unless an output
  * overlaps an input, which is allowed: the other ways write after the last
- * read); otherwise, when the
- * range is at most 4 keys per row, the groups are summed in a slot array over
- * the range -- or, for rows in no order of which a sample finds a key often,
- * in the hash table when that takes less memory, and again in the slot array
- * if it does not hold them. */
+ * read); otherwise, when the range is at most 4 keys per row, the groups are
+ * summed in a slot array over the range -- or, for rows in no order of which
+ * a sample finds a key often, in the hash table when that takes less memory,
+ * and again in the slot array if it does not hold them. */
 pq_status pq_groupby_sum(pq_ctx* ctx, pq_col key, pq_col val, int64_t* out_keys,
                          int64_t* out_sums, int64_t cap, int64_t* d_ngroups, void* stream);
 
